@@ -20,10 +20,11 @@ LIB = os.path.join(BUILD, "liblskum.so")
 PROBE = os.path.join(BUILD, "pipe_peaks")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-CUDA_SOURCES = ["lskum_kernels.cu", "lskum_kernels_mixed.cu", "lskum_api.cu", "lskum_noalloc.cu",
+CUDA_SOURCES = ["lskum_kernels.cu", "lskum_kernels_pair.cu", "lskum_kernels_mixed.cu", "lskum_api.cu", "lskum_noalloc.cu",
                 "mlp_kernels.cu"]
 HOST_SOURCES = ["lskum_setup.cpp"]
-HEADERS = ["lskum_internal.h", "lskum_kernels.cuh", "math_tables.h", "device_math.cuh"]
+HEADERS = ["lskum_internal.h", "lskum_kernels.cuh", "math_tables.h", "device_math.cuh",
+           "flux_fp64.cuh", "pair_math.cuh", "flux_pair.cuh", "pair_tables.h"]
 
 
 def _nvcc() -> str:

@@ -47,7 +47,9 @@ struct lskum_ctx {
 
     HostLayout host;
     bool mixed = false;
+    bool pairs = false;  // FP64 path: the fused flux in float pairs (gamma = 1.4)
     DevGeom g{};
+    DevGeomPair gp{};
     DevGeom32 g32{};
     Physics ph{};
     DevState st{};
@@ -137,14 +139,21 @@ cudaError_t timed(lskum_ctx* c, int cls, F&& launch) {
     return e;
 }
 
-int n_blocks(const lskum_ctx* c) { return int((c->g.n + c->block - 1) / c->block); }
+// blocks of the stage-1 flux kernel: one partial sum of the residue each
+int n_blocks(const lskum_ctx* c) {
+    if (c->pairs) return int(pair_flux_blocks(c->g, c->block));
+    return int((c->g.n + c->block - 1) / c->block);
+}
 
-// q-derivatives of the q buffer `qb` into dq[final] (FP64) or dq32[final]
-// (mixed); returns the index of the buffer holding the result.
-cudaError_t run_q_derivatives(lskum_ctx* c, int qb, int* final_buf, int64_t* launches) {
+// q-derivatives of the q buffer `qb` into dq[final] (FP64; as float pairs if
+// the pair-form flux kernel takes them) or dq32[final] (mixed); returns the
+// index of the buffer holding the result.
+cudaError_t run_q_derivatives(lskum_ctx* c, int qb, bool for_flux, int* final_buf, int64_t* launches) {
+    const bool pairs = for_flux && c->pairs;
     cudaError_t e = timed(c, kLsFirst, [&] {
         return c->mixed ? launch_ls_first_mx(c->g, c->g32, c->st.qhl[qb], c->st.dq32[0], c->block_ls, c->stream)
-                        : launch_ls_first(c->g, c->st.q[qb], c->st.dq[0], c->block_ls, c->stream);
+                        : launch_ls_first(c->g, c->st.q[qb], c->st.dq[0], pairs && c->opt.inner_iters == 0,
+                                          c->block_ls, c->stream);
     });
     if (e != cudaSuccess) return e;
     ++*launches;
@@ -157,7 +166,8 @@ cudaError_t run_q_derivatives(lskum_ctx* c, int qb, int* final_buf, int64_t* lau
             return c->mixed ? launch_ls_inner_mx(c->g, c->g32, c->st.dq32[0], c->st.dq32[cur],
                                                  c->st.dq32[next], c->block_ls, c->stream)
                             : launch_ls_inner(c->g, c->st.dq[0], c->st.dq[cur], c->st.dq[next],
-                                              c->block_ls, c->stream);
+                                              pairs && it + 1 == c->opt.inner_iters, c->block_ls,
+                                              c->stream);
         });
         if (e != cudaSuccess) return e;
         ++*launches;
@@ -174,6 +184,10 @@ cudaError_t launch_flux_any(lskum_ctx* c, int mode, int qb, int dbuf, int qout) 
     if (c->opt.flux_split)
         return launch_flux_split(mode, c->g, c->ph, c->st, c->st.q[qb], c->st.dq[dbuf],
                                  qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
+    if (c->pairs)
+        return launch_flux_pair(mode, c->g, c->gp, c->ph, c->st, c->st.q[qb],
+                                reinterpret_cast<const DQP*>(c->st.dq[dbuf]),
+                                qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
     return launch_flux(mode, c->g, c->ph, c->st, c->st.q[qb], c->st.dq[dbuf],
                        qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
 }
@@ -184,7 +198,7 @@ cudaError_t run_iteration(lskum_ctx* c, int64_t* launches) {
     int qcur = 0;
     for (int stage = 1; stage <= 4; ++stage) {
         int dbuf = 0;
-        cudaError_t e = run_q_derivatives(c, qcur, &dbuf, launches);
+        cudaError_t e = run_q_derivatives(c, qcur, true, &dbuf, launches);
         if (e != cudaSuccess) return e;
         e = timed(c, kFlux, [&] { return launch_flux_any(c, stage, qcur, dbuf, 1 - qcur); });
         if (e != cudaSuccess) return e;
@@ -281,13 +295,14 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
     c->block = o.block_size ? o.block_size : kDefaultBlock;
     c->block_ls = c->block;
     c->mixed = o.precision == LSKUM_MIXED;
+    c->pairs = !c->mixed && !o.flux_split && std::fabs(1.0 / (o.gamma - 1.0) - 2.5) < 1e-12;
     c->C = o.n_conditions;
     c->mach.assign(c->C, 0.0);
     c->alpha.assign(c->C, 0.0);
 
     // host validation and layout first: input errors are reported without a GPU
     std::string err;
-    int rc = build_layout(n, xy, normals, flags, nbr_offsets, nbr_idx, o, c->host, err);
+    int rc = build_layout(n, xy, normals, flags, nbr_offsets, nbr_idx, o, c->pairs, c->host, err);
     if (rc != LSKUM_OK) {
         delete c;
         return fail(rc, err);
@@ -334,13 +349,21 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
         return bail(e, "upload of the cloud layout");
 
     if (!c->mixed) {
-        if ((e = upload(c, &g.hdx, L.hdx)) != cudaSuccess ||
-            (e = upload(c, &g.hdy, L.hdy)) != cudaSuccess ||
-            (e = upload(c, &g.wx, L.wx)) != cudaSuccess ||
-            (e = upload(c, &g.wy, L.wy)) != cudaSuccess ||
-            (e = upload(c, &g.ws, L.ws)) != cudaSuccess ||
-            (e = upload(c, &g.wn, L.wn)) != cudaSuccess)
+        if ((e = upload(c, &g.wx, L.wx)) != cudaSuccess || (e = upload(c, &g.wy, L.wy)) != cudaSuccess)
             return bail(e, "upload of the FP64 cloud layout");
+        if (c->pairs) {
+            const float *half = nullptr, *weight = nullptr;
+            if ((e = upload(c, &half, L.half)) != cudaSuccess ||
+                (e = upload(c, &weight, L.weight)) != cudaSuccess)
+                return bail(e, "upload of the float-pair cloud layout");
+            c->gp.half = reinterpret_cast<const float4*>(half);
+            c->gp.weight = reinterpret_cast<const float4*>(weight);
+        } else if ((e = upload(c, &g.hdx, L.hdx)) != cudaSuccess ||
+                   (e = upload(c, &g.hdy, L.hdy)) != cudaSuccess ||
+                   (e = upload(c, &g.ws, L.ws)) != cudaSuccess ||
+                   (e = upload(c, &g.wn, L.wn)) != cudaSuccess) {
+            return bail(e, "upload of the FP64 cloud layout");
+        }
         std::vector<V4> lcoef(L.lc.size() / 4), lsum(L.lsum.size() / 4);
         std::memcpy(lcoef.data(), L.lc.data(), L.lc.size() * sizeof(double));
         std::memcpy(lsum.data(), L.lsum.data(), L.lsum.size() * sizeof(double));
@@ -370,7 +393,8 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
 
     DevState& st = c->st;
     const size_t N = size_t(L.n) * size_t(c->C);  // (point, condition) pairs
-    const int nb = int((L.n + 127) / 128) + 1;  // block partials when C == 1
+    // block partials when C == 1
+    const int nb = 1 + int(c->pairs ? pair_flux_blocks(g, kDefaultBlock) : (L.n + kDefaultBlock - 1) / kDefaultBlock);
     if (c->mixed) {
         if ((e = dev_alloc(c, &st.qhl[0], N)) != cudaSuccess ||
             (e = dev_alloc(c, &st.qhl[1], N)) != cudaSuccess ||
@@ -597,7 +621,7 @@ int lskum_eval_residual(lskum_ctx* c, double* R) {
     if (!c->have_state) return fail(LSKUM_ERR_STATE, "no state set");
     int dbuf = 0;
     int64_t launches = 0;
-    cudaError_t e = run_q_derivatives(c, 0, &dbuf, &launches);
+    cudaError_t e = run_q_derivatives(c, 0, true, &dbuf, &launches);
     if (e != cudaSuccess) return cuda_fail(e, "q-derivatives");
     LSKUM_CUDA(launch_flux_any(c, 0, 0, dbuf, -1));
     LSKUM_CUDA(launch_gather_v4(c->g, c->st.R, c->staging, c->stream));
@@ -615,7 +639,7 @@ int lskum_eval_q_derivatives(lskum_ctx* c, double* qx, double* qy) {
     }
     int dbuf = 0;
     int64_t launches = 0;
-    cudaError_t e = run_q_derivatives(c, 0, &dbuf, &launches);
+    cudaError_t e = run_q_derivatives(c, 0, false, &dbuf, &launches);
     if (e != cudaSuccess) return cuda_fail(e, "q-derivatives");
     if (c->mixed) {
         LSKUM_CUDA(launch_dq_to_user_mx(c->g, c->st.dq32[dbuf], c->staging8, c->stream));

@@ -35,6 +35,9 @@ struct HostLayout {
     std::vector<double> hdx, hdy;  // half of the global offsets x_j - x_i, y_j - y_i
     std::vector<double> wx, wy;    // full-stencil least-squares weights (Eq. 11)
     std::vector<double> ws, wn;    // split-stencil weights of d/ds and d/dn (Eq. 24)
+    // with `pairs`, in place of hdx, hdy, ws, wn: {hdx hi, lo, hdy hi, lo} and
+    // {ws hi, lo, wn hi, lo}, four floats a slot
+    std::vector<float> half, weight;
     // FP64 inner sweeps (Eq. 29) split as q_x = (first-order q_x) - sum_j wx_j
     // (hdx_j (qx_j - qx_i) + hdy_j (qy_j - qy_i)), likewise q_y: per slot the
     // products {wx hdx, wx hdy, wy hdx, wy hdy} (4 per slot, [slot][stride]),
@@ -47,9 +50,9 @@ struct HostLayout {
 };
 
 // Validates the caller's cloud and builds the device layout. Returns LSKUM_OK
-// or an error code with a message in `err`.
+// or an error code with a message in `err`. `pairs`: see HostLayout.
 int build_layout(int64_t n, const double* xy, const double* normals, const int8_t* flags,
-                 const int32_t* offsets, const int32_t* idx, const lskum_options& opt,
+                 const int32_t* offsets, const int32_t* idx, const lskum_options& opt, bool pairs,
                  HostLayout& out, std::string& err);
 
 void set_last_error(const std::string& msg);

@@ -31,6 +31,19 @@ struct __align__(32) D8f {
     float4 y;
 };
 
+// q-derivatives of one point as float pairs (hi + lo = the FP64 value to
+// ~2^-49), the flux kernel's input in the pair form; the size of a V8.
+struct __align__(64) DQP {
+    float4 xh, xl, yh, yl;
+};
+
+// Per-neighbour constants of the pair-form flux kernel, slot-major
+// [slot][stride], hi and lo floats interleaved.
+struct DevGeomPair {
+    const float4* half;    // half offsets {hdx hi, lo, hdy hi, lo}
+    const float4* weight;  // split-stencil weights {ws hi, lo, wn hi, lo}
+};
+
 // FP32 copies of the slot-major per-neighbour arrays (mixed precision).
 struct DevGeom32 {
     // slot-major [slot][stride], one record per neighbour entry so a kernel
@@ -122,12 +135,22 @@ __host__ __device__ __forceinline__ int64_t sidx(const DevGeom& g, int64_t d, ui
 }
 
 // Launchers (return cudaGetLastError()).
-cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, int block, cudaStream_t s);
-cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* dq_in, V8* dq_out, int block,
+// as_pairs: the result is written as DQP records (for launch_flux_pair)
+// instead of V8 ones, into the same memory.
+cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, bool as_pairs, int block,
                             cudaStream_t s);
+cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* dq_in, V8* dq_out,
+                            bool as_pairs, int block, cudaStream_t s);
 // mode 0: evaluate R only (written to st.R); mode 1..4: SSP-RK stage.
 cudaError_t launch_flux(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                         const V4* q_in, const V8* dq, V4* q_out, int block, cudaStream_t s);
+// The same for gamma = 1.4 with the neighbour pairs' work in float pairs.
+cudaError_t launch_flux_pair(int mode, const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
+                             const DevState& st, const V4* q_in, const DQP* dq, V4* q_out, int block,
+                             cudaStream_t s);
+// Threads it gives a point, and its blocks (of `block` threads) for the cloud.
+int pair_flux_lanes(const DevGeom& g);
+int64_t pair_flux_blocks(const DevGeom& g, int block);
 // The paper's four split-flux kernels + a stage kernel (ablation of launch_flux;
 // 5 launches; uses st.R as the accumulator).
 cudaError_t launch_flux_split(int mode, const DevGeom& g, const Physics& ph, const DevState& st,

@@ -63,10 +63,18 @@ inline Frame frame_of(int8_t flag, const double* nrm) {
     return {nrm[1], -nrm[0], nrm[0], nrm[1]};
 }
 
+// Two doubles as float pairs {a hi, a lo, b hi, b lo}.
+inline void split2(double a, double b, float* out) {
+    out[0] = float(a);
+    out[1] = float(a - double(out[0]));
+    out[2] = float(b);
+    out[3] = float(b - double(out[2]));
+}
+
 }  // namespace
 
 int build_layout(int64_t n, const double* xy, const double* normals, const int8_t* flags,
-                 const int32_t* off, const int32_t* idx, const lskum_options& opt,
+                 const int32_t* off, const int32_t* idx, const lskum_options& opt, bool pairs,
                  HostLayout& L, std::string& err) {
     std::ostringstream msg;
     if (n < 1 || n > kMaxPoints) {
@@ -167,12 +175,17 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
     L.nrm.assign(2 * n, 0.0);
     L.dmin.assign(n, 0.0);
     L.nbr.assign(size_t(slots) * S, 0u);
-    L.hdx.assign(size_t(slots) * S, 0.0);
-    L.hdy.assign(size_t(slots) * S, 0.0);
     L.wx.assign(size_t(slots) * S, 0.0);
     L.wy.assign(size_t(slots) * S, 0.0);
-    L.ws.assign(size_t(slots) * S, 0.0);
-    L.wn.assign(size_t(slots) * S, 0.0);
+    if (pairs) {
+        L.half.assign(size_t(slots) * S * 4, 0.0f);
+        L.weight.assign(size_t(slots) * S * 4, 0.0f);
+    } else {
+        L.hdx.assign(size_t(slots) * S, 0.0);
+        L.hdy.assign(size_t(slots) * S, 0.0);
+        L.ws.assign(size_t(slots) * S, 0.0);
+        L.wn.assign(size_t(slots) * S, 0.0);
+    }
     const bool want_lc = opt.precision == LSKUM_FP64;
     if (want_lc) {
         L.lc.assign(size_t(slots) * S * 4, 0.0);
@@ -273,18 +286,24 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
                 if (b == 3) wn *= wall_fac;
             }
             L.nbr[at] = uint32_t(L.user_to_dev[j]) | (s_code << kIndexBits) | (n_code << (kIndexBits + 2));
-            L.hdx[at] = 0.5 * dx[k];
-            L.hdy[at] = 0.5 * dy[k];
+            const double hx = 0.5 * dx[k], hy = 0.5 * dy[k];
             L.wx[at] = wt[k] * (dx[k] * syy - dy[k] * sxy) / det;
             L.wy[at] = wt[k] * (dy[k] * sxx - dx[k] * sxy) / det;
-            L.ws[at] = ws;
-            L.wn[at] = wn;
+            if (pairs) {
+                split2(hx, hy, &L.half[4 * at]);
+                split2(ws, wn, &L.weight[4 * at]);
+            } else {
+                L.hdx[at] = hx;
+                L.hdy[at] = hy;
+                L.ws[at] = ws;
+                L.wn[at] = wn;
+            }
             if (want_lc) {
                 double* c4 = &L.lc[4 * at];
-                c4[0] = L.wx[at] * L.hdx[at];
-                c4[1] = L.wx[at] * L.hdy[at];
-                c4[2] = L.wy[at] * L.hdx[at];
-                c4[3] = L.wy[at] * L.hdy[at];
+                c4[0] = L.wx[at] * hx;
+                c4[1] = L.wx[at] * hy;
+                c4[2] = L.wy[at] * hx;
+                c4[3] = L.wy[at] * hy;
                 for (int m = 0; m < 4; ++m) L.lsum[4 * d + m] += c4[m];
             }
         }

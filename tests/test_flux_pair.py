@@ -1,0 +1,60 @@
+"""The float-pair form of the split-flux differences (csrc/flux_pair.cuh) on the
+CPU, against binary128 and a plain double evaluation, and its tables against
+their generator."""
+
+import importlib.util
+import os
+import platform
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2108_07031_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def checker(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("flux_pair") / "check")
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-o", exe,
+                    os.path.join(ROOT, "tests", "flux_pair", "check_flux_pair.cpp")]
+                   + (["-lquadmath"] if platform.machine() == "x86_64" else []), check=True)
+
+    def run(mach, log2_step, pairs=2000):
+        out = subprocess.run([exe, str(mach), str(log2_step), str(pairs)], check=True,
+                             capture_output=True, text=True).stdout.split()
+        return int(out[0]), [float(v) for v in out[1:5]], [float(v) for v in out[5:9]]
+    return run
+
+
+@pytest.mark.parametrize("mach", [0.0, 0.3, 0.85, 2.0])
+@pytest.mark.parametrize("log2_step", [-20, -12, -8, -7])
+def test_difference_error(checker, mach, log2_step):
+    """About a hundred pair operations of 2^-47 each stand behind a component:
+    2^-43 of dG in the 2-norm; and no further off than the double evaluation,
+    which is left with 2^-51.5 / step (in still air state 0 has no momentum to
+    cancel, so double has nothing to lose there)."""
+    taken, err, err64 = checker(mach, log2_step)
+    # beyond Mach 1 ln(rho beta^2.5) moves by many times the step
+    assert taken == 2000 or (log2_step == -7 and taken > 1000)
+    assert max(err) < 2.0 ** -43
+    assert mach == 0.0 or all(a <= b for a, b in zip(err, err64))
+
+
+@pytest.mark.parametrize("mach, log2_step", [(0.63, -1), (40.0, -20)])
+def test_large_steps_and_states_out_of_range_are_left_out(checker, mach, log2_step):
+    """Steps over the limits, and |S| beyond the table of Phi (most pairs at
+    Mach 40): the form refuses them."""
+    assert checker(mach, log2_step)[0] < 60
+
+
+def test_tables_match_their_generator(tmp_path):
+    pytest.importorskip("mpmath")
+    spec = importlib.util.spec_from_file_location("gen_pair_tables",
+                                                  os.path.join(CSRC, "gen_pair_tables.py"))
+    gen = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(gen)
+    out = tmp_path / "pair_tables.h"
+    gen.main(str(out))
+    with open(os.path.join(CSRC, "pair_tables.h")) as f:
+        assert out.read_text() == f.read()
