@@ -145,8 +145,8 @@ int n_blocks(const lskum_ctx* c) {
     return int((c->g.n + c->block - 1) / c->block);
 }
 
-// q-derivatives of the q buffer `qb` into dq[final] (FP64; as float pairs if
-// the pair-form flux kernel takes them) or dq32[final] (mixed); returns the
+// q-derivatives of the q buffer `qb` into dq[final] (FP64; for_flux: in float
+// pairs if the flux kernel takes them so) or dq32[final] (mixed); returns the
 // index of the buffer holding the result.
 cudaError_t run_q_derivatives(lskum_ctx* c, int qb, bool for_flux, int* final_buf, int64_t* launches) {
     const bool pairs = for_flux && c->pairs;

@@ -31,55 +31,53 @@ namespace lskum {
 namespace {
 
 // ----------------------------------------------------------- q-derivatives
+//
+// Four threads a (point, condition), one for each component of q: a gathered
+// record is one coalesced read of its four threads where a thread of its own
+// for each point made 32 scattered ones a load, and a small cloud fills four
+// times the SMs: 5,120 points 15 -> 10 us the first-order sweep, 20 -> 14 an
+// inner one; at 0.6M points and more both forms are bound by the FP64 pipe
+// (190 and 285 us). A component's sum keeps the slot order.
 
-// Stores the derivatives of one point: FP64, or as float pairs for the
-// pair-form flux kernel (hi and lo each rounded to nearest).
+// Stores a component's derivatives: FP64, or as float pairs for the pair-form
+// flux kernel (hi and lo each rounded to nearest).
 template <bool PAIRS>
-__device__ __forceinline__ void store_dq(V8* p, const double x[4], const double y[4]) {
+__device__ __forceinline__ void store_dq(V8* p, const int m, const double x, const double y) {
     if (PAIRS) {
-        float xh[4], xl[4], yh[4], yl[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            xh[m] = __double2float_rn(x[m]);
-            xl[m] = __double2float_rn(x[m] - double(xh[m]));
-            yh[m] = __double2float_rn(y[m]);
-            yl[m] = __double2float_rn(y[m] - double(yh[m]));
-        }
-        *reinterpret_cast<DQP*>(p) = DQP{make_float4(xh[0], xh[1], xh[2], xh[3]),
-                                         make_float4(xl[0], xl[1], xl[2], xl[3]),
-                                         make_float4(yh[0], yh[1], yh[2], yh[3]),
-                                         make_float4(yl[0], yl[1], yl[2], yl[3])};
+        float4 v;
+        v.x = __double2float_rn(x);
+        v.y = __double2float_rn(x - double(v.x));
+        v.z = __double2float_rn(y);
+        v.w = __double2float_rn(y - double(v.z));
+        reinterpret_cast<DQP*>(p)->c[m] = v;
     } else {
-        V8 o;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            o.x[m] = x[m];
-            o.y[m] = y[m];
-        }
-        *p = o;
+        p->x[m] = x;
+        p->y[m] = y;
     }
 }
 
 template <int BLOCK, bool PAIRS>
 __global__ void __launch_bounds__(BLOCK) k_ls_first(const DevGeom g, const V4* __restrict__ q,
                                                     V8* __restrict__ dq) {
-    const int64_t t = int64_t(blockIdx.x) * BLOCK + threadIdx.x;  // (point, condition)
+    const int64_t t = (int64_t(blockIdx.x) * BLOCK + threadIdx.x) / 4;  // (point, condition)
+    const int m = threadIdx.x % 4;
     const int64_t d = t >> g.cshift;
     const uint32_t cc = uint32_t(t) & g.cmask;
     if (d >= g.n) return;
-    const V4 qi = ld4(q + t);
-    double ax[4] = {0, 0, 0, 0}, ay[4] = {0, 0, 0, 0};
+    const double* qm = reinterpret_cast<const double*>(q) + m;
+    const double qi = qm[4 * t];
+    double ax = 0.0, ay = 0.0;
     const int c = g.cnt[d];
+#pragma unroll 4
     for (int k = 0; k < c; ++k) {
         const int64_t at = int64_t(k) * g.stride + d;
         const uint32_t j = g.nbr[at] & kIndexMask;
         const double wx = g.wx[at], wy = g.wy[at];
-        const V4 qj = ld4(q + sidx(g, j, cc));
-        const double dq0 = qj.a - qi.a, dq1 = qj.b - qi.b, dq2 = qj.c - qi.c, dq3 = qj.d - qi.d;
-        ax[0] += wx * dq0; ax[1] += wx * dq1; ax[2] += wx * dq2; ax[3] += wx * dq3;
-        ay[0] += wy * dq0; ay[1] += wy * dq1; ay[2] += wy * dq2; ay[3] += wy * dq3;
+        const double e = qm[4 * sidx(g, j, cc)] - qi;
+        ax += wx * e;
+        ay += wy * e;
     }
-    store_dq<PAIRS>(dq + t, ax, ay);
+    store_dq<PAIRS>(dq + t, m, ax, ay);
 }
 
 // One Jacobi sweep of Eq. 29. With dq~_j = (q_j - q_i) - (hdx_j (qx_j - qx_i)
@@ -95,32 +93,27 @@ template <int BLOCK, bool PAIRS>
 __global__ void __launch_bounds__(BLOCK) k_ls_inner(const DevGeom g, const V8* __restrict__ dq_first,
                                                     const V8* __restrict__ din,
                                                     V8* __restrict__ dout) {
-    const int64_t t = int64_t(blockIdx.x) * BLOCK + threadIdx.x;  // (point, condition)
+    const int64_t t = (int64_t(blockIdx.x) * BLOCK + threadIdx.x) / 4;  // (point, condition)
+    const int m = threadIdx.x % 4;
     const int64_t d = t >> g.cshift;
     const uint32_t cc = uint32_t(t) & g.cmask;
     if (d >= g.n) return;
-    double ax[4] = {0, 0, 0, 0}, ay[4] = {0, 0, 0, 0};
+    double ax = 0.0, ay = 0.0;
     const int c = g.cnt[d];
+#pragma unroll 4
     for (int k = 0; k < c; ++k) {
         const int64_t at = int64_t(k) * g.stride + d;
         const uint32_t j = g.nbr[at] & kIndexMask;
         const V4 p = g.lcoef[at];
-        const V8 dj = din[sidx(g, j, cc)];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            ax[m] = fma(p.a, dj.x[m], fma(p.b, dj.y[m], ax[m]));
-            ay[m] = fma(p.c, dj.x[m], fma(p.d, dj.y[m], ay[m]));
-        }
+        const V8* dj = din + sidx(g, j, cc);
+        const double x = dj->x[m], y = dj->y[m];
+        ax = fma(p.a, x, fma(p.b, y, ax));
+        ay = fma(p.c, x, fma(p.d, y, ay));
     }
     const V4 S = g.lsum[d];
-    const V8 di = din[t];
-    const V8 f = dq_first[t];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        ax[m] = f.x[m] - (ax[m] - fma(S.a, di.x[m], S.b * di.y[m]));
-        ay[m] = f.y[m] - (ay[m] - fma(S.c, di.x[m], S.d * di.y[m]));
-    }
-    store_dq<PAIRS>(dout + t, ax, ay);
+    const double xi = din[t].x[m], yi = din[t].y[m];
+    store_dq<PAIRS>(dout + t, m, dq_first[t].x[m] - (ax - fma(S.a, xi, S.b * yi)),
+                    dq_first[t].y[m] - (ay - fma(S.c, xi, S.d * yi)));
 }
 
 // ------------------------------------------------------- flux residual + RK
@@ -507,7 +500,7 @@ inline unsigned grid_nc(const DevGeom& g, int block) { return grid_for(g.n << g.
 
 cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, bool as_pairs, int block,
                             cudaStream_t s) {
-    const unsigned grid = grid_nc(g, block);
+    const unsigned grid = grid_for((g.n << g.cshift) * 4, block);
     if (block == 256) {
         if (as_pairs) k_ls_first<256, true><<<grid, 256, 0, s>>>(g, q, dq);
         else k_ls_first<256, false><<<grid, 256, 0, s>>>(g, q, dq);
@@ -520,7 +513,7 @@ cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, bool as_pairs
 
 cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* din, V8* dout, bool as_pairs,
                             int block, cudaStream_t s) {
-    const unsigned grid = grid_nc(g, block);
+    const unsigned grid = grid_for((g.n << g.cshift) * 4, block);
     if (block == 256) {
         if (as_pairs) k_ls_inner<256, true><<<grid, 256, 0, s>>>(g, dq_first, din, dout);
         else k_ls_inner<256, false><<<grid, 256, 0, s>>>(g, dq_first, din, dout);

@@ -32,9 +32,10 @@ struct __align__(32) D8f {
 };
 
 // q-derivatives of one point as float pairs (hi + lo = the FP64 value to
-// ~2^-49), the flux kernel's input in the pair form; the size of a V8.
+// ~2^-49), the flux kernel's input in the pair form: per component {q_x hi, lo,
+// q_y hi, lo}. The size of a V8.
 struct __align__(64) DQP {
-    float4 xh, xl, yh, yl;
+    float4 c[4];
 };
 
 // Per-neighbour constants of the pair-form flux kernel, slot-major

@@ -55,25 +55,8 @@ __device__ __forceinline__ double widen(const float x) {
 
 __device__ __forceinline__ double join(const Pf a) { return widen(a.h) + widen(a.l); }
 
-__device__ __forceinline__ Pf pair_of(const float4& h, const float4& l, const int m) {
-    return m == 0 ? Pf{h.x, l.x} : m == 1 ? Pf{h.y, l.y} : m == 2 ? Pf{h.z, l.z} : Pf{h.w, l.w};
-}
-
-// Adds a point's classes, given in `sum` by each of its LANES threads (or one
-// after the other by its only one), into the first thread's `acc`.
-template <int LANES, int N>
-__device__ __forceinline__ void gather_classes(Pf acc[N], const int part) {
-    if (LANES > 1) {
-#pragma unroll
-        for (int r = 1; r < LANES; ++r)
-#pragma unroll
-            for (int m = 0; m < N; ++m) {
-                const Pf o = {__shfl_down_sync(0xffffffffu, acc[m].h, r),
-                              __shfl_down_sync(0xffffffffu, acc[m].l, r)};
-                if (part == 0) acc[m] = add(acc[m], o);
-            }
-    }
-}
+__device__ __forceinline__ Pf dx_of(const float4& c) { return Pf{c.x, c.y}; }
+__device__ __forceinline__ Pf dy_of(const float4& c) { return Pf{c.z, c.w}; }
 
 // ws dGs + wn dGn of entry k of point d in FP64, in the point's frame: what
 // k_flux adds for that entry.
@@ -99,10 +82,10 @@ __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& 
         hy = join(Pf{hp.z, hp.w});
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            vi.x[m] = join(pair_of(di.xh, di.xl, m));
-            vi.y[m] = join(pair_of(di.yh, di.yl, m));
-            vj.x[m] = join(pair_of(dj.xh, dj.xl, m));
-            vj.y[m] = join(pair_of(dj.yh, dj.yl, m));
+            vi.x[m] = join(dx_of(di.c[m]));
+            vi.y[m] = join(dy_of(di.c[m]));
+            vj.x[m] = join(dx_of(dj.c[m]));
+            vj.y[m] = join(dy_of(dj.c[m]));
         }
     }
     if (!modified_states(second, hx, hy, vj, vi, tj, t0)) return;
@@ -170,10 +153,10 @@ __device__ __forceinline__ uint32_t entries_pair(const DevGeom& g, const DevGeom
         if (second) {
             hp = gp.half[at];
             dj = dq[jt];
-            f0 -= hp.x * (dj.xh.x - P.dq.xh.x) + hp.z * (dj.yh.x - P.dq.yh.x);
-            f1 -= hp.x * (dj.xh.y - P.dq.xh.y) + hp.z * (dj.yh.y - P.dq.yh.y);
-            f2 -= hp.x * (dj.xh.z - P.dq.xh.z) + hp.z * (dj.yh.z - P.dq.yh.z);
-            f3 -= hp.x * (dj.xh.w - P.dq.xh.w) + hp.z * (dj.yh.w - P.dq.yh.w);
+            f0 -= hp.x * (dj.c[0].x - P.dq.c[0].x) + hp.z * (dj.c[0].z - P.dq.c[0].z);
+            f1 -= hp.x * (dj.c[1].x - P.dq.c[1].x) + hp.z * (dj.c[1].z - P.dq.c[1].z);
+            f2 -= hp.x * (dj.c[2].x - P.dq.c[2].x) + hp.z * (dj.c[2].z - P.dq.c[2].z);
+            f3 -= hp.x * (dj.c[3].x - P.dq.c[3].x) + hp.z * (dj.c[3].z - P.dq.c[3].z);
         }
         // a step well over the limits is not taken through the pair arithmetic
         // to find that out: d(ln beta), dS and d(q1 + |S|^2) in floats
@@ -188,8 +171,8 @@ __device__ __forceinline__ uint32_t entries_pair(const DevGeom& g, const DevGeom
             const Pf hx = {hp.x, hp.y}, hy = {hp.z, hp.w};
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                const Pf c0 = add(mul(hx, pair_of(P.dq.xh, P.dq.xl, m)), mul(hy, pair_of(P.dq.yh, P.dq.yl, m)));
-                const Pf cj = add(mul(hx, pair_of(dj.xh, dj.xl, m)), mul(hy, pair_of(dj.yh, dj.yl, m)));
+                const Pf c0 = add(mul(hx, dx_of(P.dq.c[m])), mul(hy, dy_of(P.dq.c[m])));
+                const Pf cj = add(mul(hx, dx_of(dj.c[m])), mul(hy, dy_of(dj.c[m])));
                 b[m] = sub(b[m], c0);
                 dd[m] = sub(dd[m], sub(cj, c0));
             }
@@ -275,7 +258,16 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
             for (int m = 0; m < 4; ++m) acc[m] = LANES == 1 ? add(acc[m], sum[m]) : sum[m];
         }
     }
-    gather_classes<LANES, 4>(acc, part);
+    if (LANES > 1) {
+#pragma unroll
+        for (int r = 1; r < LANES; ++r)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const Pf o = {__shfl_down_sync(0xffffffffu, acc[m].h, r),
+                              __shfl_down_sync(0xffffffffu, acc[m].l, r)};
+                if (part == 0) acc[m] = add(acc[m], o);
+            }
+    }
     double R[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) R[m] = double(acc[m].h) + double(acc[m].l);
