@@ -7,11 +7,8 @@
 // (Adam master copy) and in BF16 (W) for the GEMMs;
 // activations are stored FP32 (for tanh') and BF16 (GEMM input).
 //
-// GEMM: C[M x N] = A[M x K] B[K x N], A and B BF16 in global memory with
-// arbitrary element strides (so the forward X W^T, the backward dZ W and
-// the weight gradient dZ^T X all use one kernel), staged through shared
-// memory as A[m][k] and B[n][k] (k contiguous), 64 x 64 tiles per block of
-// four warps, mma.sync m16n8k16 (bf16 x bf16 -> f32).
+// A prediction is one kernel (k_forward), loss and gradients four: k_forward,
+// k_backward, k_weight_grads, k_reduce_grads. Every sum has a fixed order.
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -27,9 +24,6 @@
 
 namespace mlpk {
 
-constexpr int kTile = 64;
-constexpr int kKt = 32;             // k per shared-memory stage
-constexpr int kSmemPad = 8;         // bf16 padding per row (bank spread)
 constexpr int kLayers = LSKUM_MLP_LAYERS;
 constexpr int kWidth = LSKUM_MLP_WIDTH;
 constexpr int kIn = LSKUM_MLP_IN_PADDED;
@@ -38,9 +32,12 @@ constexpr int kOut = LSKUM_MLP_OUT;
 __host__ __device__ inline int layer_in(int l) { return l == 0 ? kIn : kWidth; }
 __host__ __device__ inline int layer_out(int l) { return l == kLayers - 1 ? kOut : kWidth; }
 
-__device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16* p) {
-    return *reinterpret_cast<const uint32_t*>(p);
-}
+// Offsets of W_l and b_l in the flat parameter vector, and the BF16 copies.
+struct LayerPtrs {
+    int64_t w_off[kLayers];
+    int64_t b_off[kLayers];
+    __nv_bfloat16* W[kLayers];
+};
 
 __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
     asm volatile(
@@ -50,172 +47,15 @@ __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-enum Epilogue { kStoreF32 = 0, kBiasTanh = 1, kBiasLinear = 2 };
-
-// C = A B with A(m, k) = A[m * sam + k * sak], B(k, n) = B[k * sbk + n * sbn].
-// Epilogue kBiasTanh: Zf = C + bias[n], Af = tanh(Zf), Ab = bf16(Af);
-// kBiasLinear: Cf = C + bias[n]; kStoreF32: Cf = C. Row-major outputs with
-// leading dimension ldc.
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm_bf16(const __nv_bfloat16* __restrict__ A, int64_t sam,
-                                                   int64_t sak, const __nv_bfloat16* __restrict__ B,
-                                                   int64_t sbk, int64_t sbn, int M, int N, int K,
-                                                   const float* __restrict__ bias,
-                                                   float* __restrict__ Cf,
-                                                   __nv_bfloat16* __restrict__ Cb, int64_t ldc,
-                                                   int kchunk) {
-    __shared__ __align__(16) __nv_bfloat16 As[kTile][kKt + kSmemPad];
-    __shared__ __align__(16) __nv_bfloat16 Bs[kTile][kKt + kSmemPad];
-    const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;  // warp tile origin
-    const int grp = lane >> 2, tig = lane & 3;
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
-    const __nv_bfloat16 zero = __float2bfloat16(0.f);
-    const bool a_kfast = sak == 1, b_kfast = sbk == 1;
-    // split-K: block z reduces k in [z kchunk, (z+1) kchunk) into its own
-    // slice of Cf (summed afterwards in slice order)
-    const int kbeg = blockIdx.z * kchunk;
-    const int kend = min(K, kbeg + kchunk);
-    if (EPI == kStoreF32) Cf += int64_t(blockIdx.z) * M * ldc;
-    for (int k0 = kbeg; k0 < kend; k0 += kKt) {
-        // stage: 64 x 32 elements of each operand, 16 per thread; consecutive
-        // threads walk the operand's contiguous dimension (coalesced loads)
-        for (int e = tid; e < kTile * kKt; e += 128) {
-            const int r = a_kfast ? e / kKt : e % kTile;
-            const int kk = a_kfast ? e % kKt : e / kTile;
-            const int gm = m0 + r, gk = k0 + kk;
-            As[r][kk] = (gm < M && gk < kend) ? A[gm * sam + gk * sak] : zero;
-        }
-        for (int e = tid; e < kTile * kKt; e += 128) {
-            const int r = b_kfast ? e / kKt : e % kTile;
-            const int kk = b_kfast ? e % kKt : e / kTile;
-            const int gn = n0 + r, gk = k0 + kk;
-            Bs[r][kk] = (gn < N && gk < kend) ? B[gk * sbk + gn * sbn] : zero;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < kKt; ks += 16) {
-            uint32_t af[2][4], bfr[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int row = wm + i * 16 + grp;
-                const int col = ks + tig * 2;
-                af[i][0] = ld_pair(&As[row][col]);
-                af[i][1] = ld_pair(&As[row + 8][col]);
-                af[i][2] = ld_pair(&As[row][col + 8]);
-                af[i][3] = ld_pair(&As[row + 8][col + 8]);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int n = wn + j * 8 + grp;
-                const int k = ks + tig * 2;
-                bfr[j][0] = ld_pair(&Bs[n][k]);
-                bfr[j][1] = ld_pair(&Bs[n][k + 8]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16_16816(acc[i][j], af[i], bfr[j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int m = m0 + wm + i * 16 + grp + ((r & 2) ? 8 : 0);
-                const int n = n0 + wn + j * 8 + tig * 2 + (r & 1);
-                if (m >= M || n >= N) continue;
-                float v = acc[i][j][r];
-                if (EPI != kStoreF32) v += bias[n];
-                if (EPI == kBiasTanh) {
-                    const float a = tanhf(v);
-                    Cf[int64_t(m) * ldc + n] = a;
-                    Cb[int64_t(m) * ldc + n] = __float2bfloat16(a);
-                } else {
-                    Cf[int64_t(m) * ldc + n] = v;
-                }
-            }
-}
-
-// Narrow output layer, C(m, n) = sum_k X(m, k) W(n, k) + bias(n) for N <=
-// kNarrowMax outputs (the network's 4-wide last layer): one warp per row of
-// X, each lane a 16-byte chunk of eight k per step (a row of 256 is one
-// coalesced 512-byte read), W staged once per block in shared memory, FP32
-// accumulation of the exact BF16 products, a butterfly sum over the lanes.
-// The tiled GEMMs would leave 60 of their 64 (or 124 of 128) columns idle.
-// Requirements (checked by the caller): K a multiple of 8, X rows and W
-// 16-byte aligned, N <= kNarrowMax, N x K <= kNarrowW.
-constexpr int kNarrowMax = 8;
-constexpr int kNarrowW = 4096;  // bf16 elements of W in shared memory (8 KB)
-constexpr int kNarrowRows = 8;  // rows (warps) per block
-
-__global__ void __launch_bounds__(32 * kNarrowRows) k_gemm_narrow(
-    const __nv_bfloat16* __restrict__ X, int64_t sxm, const __nv_bfloat16* __restrict__ W, int M,
-    int N, int K, const float* __restrict__ bias, float* __restrict__ C, int64_t ldc) {
-    __shared__ __align__(16) __nv_bfloat16 Ws[kNarrowW];
-    const int tid = threadIdx.x, lane = tid & 31;
-    for (int e = tid * 8; e < N * K; e += 32 * kNarrowRows * 8)
-        *reinterpret_cast<uint4*>(&Ws[e]) = *reinterpret_cast<const uint4*>(W + e);
-    __syncthreads();
-    const int m = blockIdx.x * kNarrowRows + (tid >> 5);
-    if (m >= M) return;
-    float acc[kNarrowMax];
-#pragma unroll
-    for (int n = 0; n < kNarrowMax; ++n) acc[n] = 0.f;
-    const __nv_bfloat16* x = X + int64_t(m) * sxm;
-    for (int k0 = lane * 8; k0 < K; k0 += 256) {
-        const uint4 xv = *reinterpret_cast<const uint4*>(x + k0);
-        const __nv_bfloat162* xp = reinterpret_cast<const __nv_bfloat162*>(&xv);
-#pragma unroll
-        for (int n = 0; n < kNarrowMax; ++n) {
-            if (n < N) {
-                const uint4 wv = *reinterpret_cast<const uint4*>(&Ws[n * K + k0]);
-                const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float2 xf = __bfloat1622float2(xp[q]);
-                    const float2 wf = __bfloat1622float2(wp[q]);
-                    acc[n] = fmaf(xf.x, wf.x, acc[n]);
-                    acc[n] = fmaf(xf.y, wf.y, acc[n]);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < kNarrowMax; ++n)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], o);
-    if (lane < N) {
-        float v = acc[0];
-#pragma unroll
-        for (int n = 1; n < kNarrowMax; ++n)
-            if (lane == n) v = acc[n];
-        C[int64_t(m) * ldc + lane] = v + bias[lane];
-    }
-}
-
-// Pipelined GEMM for the aligned, large shapes: 128 x 128 tiles per block of
-// eight warps (each 64 x 32), k in stages of 32 moved global -> shared by
-// cp.async (16-byte chunks, three stages in flight), operand fragments by
-// ldmatrix -- plain for an operand whose contraction index is contiguous in
-// memory (X and W in the forward pass), transposed for one whose row index
-// is (dZ^T and X in the weight gradient, W in dZ W) -- and the same
-// mma.sync m16n8k16 and epilogues as k_gemm_bf16. Requirements (checked by
-// the caller): the contiguous dimension of each operand a multiple of 8
-// elements with 16-byte aligned rows, kchunk a multiple of 32.
+// Pipelined GEMM tile: 128 x 128 outputs a block of eight warps (each 64 x 32),
+// k in stages of 32 moved global -> shared by cp.async (16-byte chunks, three
+// stages in flight), operand fragments by ldmatrix -- plain for an operand whose
+// contraction index is contiguous in memory, transposed for one whose row index
+// is (dZ^T and X in the weight gradient) -- and mma.sync m16n8k16. The
+// contiguous dimension of each operand is a multiple of 8 elements with
+// 16-byte aligned rows.
 constexpr int kTB = 128;
 constexpr int kTK = 32;
-static_assert(kTK == kKt, "split-K slices hold whole k stages of both GEMM kernels");
 constexpr int kStages = 3;
 
 template <bool KFAST>
@@ -255,24 +95,17 @@ constexpr size_t tc_smem_bytes(bool ak, bool bk) {
                   (bk ? TileGeo<true>::elems : TileGeo<false>::elems));
 }
 
-template <int EPI, bool AK, bool BK>
-__global__ void __launch_bounds__(256) k_gemm_bf16_tc(const __nv_bfloat16* __restrict__ A, int64_t sam,
-                                                      int64_t sak, const __nv_bfloat16* __restrict__ B,
-                                                      int64_t sbk, int64_t sbn, int M, int N, int K,
-                                                      const float* __restrict__ bias,
-                                                      float* __restrict__ Cf,
-                                                      __nv_bfloat16* __restrict__ Cb, int64_t ldc,
-                                                      int kchunk) {
+template <bool AK, bool BK>
+__device__ __forceinline__ void gemm_tc_block(const __nv_bfloat16* __restrict__ A, int64_t sam, int64_t sak,
+                                              const __nv_bfloat16* __restrict__ B, int64_t sbk, int64_t sbn,
+                                              int M, int N, int kbeg, int kend, int m0, int n0,
+                                              float* __restrict__ Cf, int64_t ldc) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(smem_raw);
     __nv_bfloat16* sB = sA + kStages * TileGeo<AK>::elems;
-    const int m0 = blockIdx.y * kTB, n0 = blockIdx.x * kTB;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = (warp >> 2) * 64, wn = (warp & 3) * 32;
-    const int kbeg = blockIdx.z * kchunk;
-    const int kend = min(K, kbeg + kchunk);
     const int ktiles = kend > kbeg ? (kend - kbeg + kTK - 1) / kTK : 0;
-    if (EPI == kStoreF32) Cf += int64_t(blockIdx.z) * M * ldc;
 
     // one stage: 512 16-byte chunks of each operand tile, two per thread
     auto load_stage = [&](int stage, int kt) {
@@ -373,42 +206,62 @@ __global__ void __launch_bounds__(256) k_gemm_bf16_tc(const __nv_bfloat16* __res
                 const int m = m0 + wm + i * 16 + grp + ((r & 2) ? 8 : 0);
                 const int n = n0 + wn + j * 8 + tig * 2 + (r & 1);
                 if (m >= M || n >= N) continue;
-                float v = acc[i][j][r];
-                if (EPI != kStoreF32) v += bias[n];
-                if (EPI == kBiasTanh) {
-                    const float t = tanhf(v);
-                    Cf[int64_t(m) * ldc + n] = t;
-                    Cb[int64_t(m) * ldc + n] = __float2bfloat16(t);
-                } else {
-                    Cf[int64_t(m) * ldc + n] = v;
-                }
+                Cf[int64_t(m) * ldc + n] = acc[i][j][r];
             }
 }
 
-// ------------------------------------------------- tcgen05 forward GEMM
-// Z = X W^T + b (tanh or linear epilogue) of a hidden layer (256 outputs) on
-// the fifth-generation tensor cores. One CTA of eight warps per 128-row tile
-// of X and 128-column half of the outputs: it stages X[m0:m0+128, 0:K] and
-// W[n0:n0+128, 0:K] (K <= 256: at most 2 x 64 KB) in shared memory with
-// cp.async in K stages of 64 (one copy group each), and as each stage lands
-// one thread issues its four tcgen05.mma (M 128, N 128, K 16, BF16 x BF16 ->
-// FP32) into a 128-column accumulator in tensor memory, so the MMAs of a
-// stage overlap the copies of the next; the last commit arrives on an
-// mbarrier, and each warp reads a 32-lane x 64-column quarter of the
-// accumulator back with tcgen05.ld for the epilogue (warp w: lanes 32 (w mod
-// 4) .., columns 64 (w div 4) ..).
+// ------------------------------------------------- fused forward pass
+// All six layers of a 128-row tile in one CTA on the fifth-generation tensor
+// cores: the activations stay in shared memory as BF16 A operands, the weights
+// stream from L2 through a ring of four 32 KB slots (64 of a layer's 256 k
+// each, laid out beforehand as the operand image, one bulk copy a slot), and
+// a layer's products accumulate in 256 columns of tensor memory, two layers'
+// accumulators side by side. Eight warps turn the accumulators into the next
+// layer's operand (bias, tanh, BF16), 64 columns at a time; the MMAs of those
+// 64 k start as soon as they are written, so they run under the tanh of the
+// next 64. One warp issues the MMAs, one the copies. The 4-wide output layer
+// is FP32 FMAs on the same BF16 values, in the last epilogue.
 //
-// Shared-memory operand layout: the no-swizzle K-major canonical form of the
-// matrix descriptors: core matrices of 8 rows x 16 bytes (8 BF16 along K)
-// stored as 128 contiguous bytes; core matrix (r/8, k/8) of an operand at
-// byte (r/8) SBO + (k/8) LBO with LBO = 128 (next core matrix along K) and
-// SBO = 16 K (next 8-row group). One MMA reads two core matrices along K, so
-// consecutive MMAs advance both descriptors' start by 256 bytes.
-constexpr int kUmmaM = 128, kUmmaN = 128, kUmmaK = 16, kUmmaStageK = 64, kUmmaThreads = 256;
-constexpr int kUmmaOut = 256;  // outputs of a hidden layer (two CTAs' halves)
+// What bounds it: tanhf, 163,840 a tile on an SM's FP32 pipes (~25 instructions
+// each); the MMAs of a tile are 68 MFLOP x 2, 11 us at the SM's share of the
+// BF16 rate, mostly hidden. A launch per layer wrote and re-read the
+// activations (1.5 KB a row and layer) and filled the chip for 2 us of work:
+// 16,384 samples 176 us a prediction, now 49 (27 in the kernel).
+//
+// Operand layout: the no-swizzle K-major canonical form of the matrix
+// descriptors: core matrices of 8 rows x 16 bytes (8 BF16 along K) as 128
+// contiguous bytes, neighbours along K 128 bytes apart (LBO), 8-row groups SBO
+// bytes apart; one MMA (K 16) reads two core matrices along K.
+constexpr int kFwdRows = 128;               // rows of a tile (MMA M)
+constexpr int kFwdSlots = 4;                // weight ring
+constexpr int kFwdSlotBytes = 256 * 64 * 2; // 256 outputs x 64 k
+constexpr int kFwdIn0Bytes = 256 * 32 * 2;  // the first layer's one chunk
+constexpr int kFwdChunks = 1 + 4 * 4;       // chunks of a tile: layer 0, then 4 each of 4 layers
+constexpr int kFwdEpi = 256;                // epilogue threads
+constexpr int kFwdThreads = kFwdEpi + 64;   // and the MMA and the copy warp
+constexpr int kFwdABytes = kFwdRows * 256 * 2;
+constexpr int kFwdHidden = kLayers - 1;
+// shared memory: A, ring, biases, output layer (weights as float4 a column), row partials, barriers
+constexpr int kFwdOffRing = kFwdABytes;
+constexpr int kFwdOffBias = kFwdOffRing + kFwdSlots * kFwdSlotBytes;
+constexpr int kFwdOffW5 = kFwdOffBias + kFwdHidden * 256 * 4;
+constexpr int kFwdOffPart = kFwdOffW5 + 256 * 16;
+constexpr int kFwdOffBar = kFwdOffPart + kFwdRows * 16;
+constexpr int kFwdSmem = kFwdOffBar + 128;
+static_assert(kFwdSmem <= 227 * 1024, "one CTA's shared memory");
 
-__host__ __device__ constexpr size_t umma_smem_bytes(int K) {
-    return size_t(kUmmaM + kUmmaN) * size_t(K) * 2 + 16;  // A, B, mbarrier, TMEM address
+// Byte offset of W_l(n, k) in the operand images, one layer after the other.
+__host__ __device__ inline int64_t packed_offset(int l, int n, int k) {
+    if (l == 0) return (n / 8) * 512 + (k / 8) * 128 + (n % 8) * 16 + (k % 8) * 2;
+    return kFwdIn0Bytes + int64_t(l - 1) * 4 * kFwdSlotBytes + (k / 64) * kFwdSlotBytes + (n / 8) * 1024 +
+           (k % 64 / 8) * 128 + (n % 8) * 16 + (k % 8) * 2;
+}
+
+// The backward pass's images: W_l transposed (row k, contraction over n) of
+// layers 4, 3, 2, 1 in the order it takes them.
+__host__ __device__ inline int64_t packed_offset_t(int l, int n, int k) {
+    return int64_t(kLayers - 2 - l) * 4 * kFwdSlotBytes + (n / 64) * kFwdSlotBytes + (k / 8) * 1024 +
+           (n % 64 / 8) * 128 + (k % 8) * 16 + (n % 8) * 2;
 }
 
 // SM100 shared-memory matrix descriptor: bits [0,14) start address >> 4,
@@ -426,11 +279,11 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
 }
 
-// Waits for phase `parity` of the mbarrier at shared address `bar`, polling
-// at most `limit` times (with a short sleep between polls); false when the
-// limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int limit) {
-    for (int i = 0; i < limit; ++i) {
+// Waits for phase `parity` of the mbarrier at shared address `bar`, polling a
+// limited number of times (about half a second; the waits here take
+// microseconds); false when the limit ran out.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    for (int i = 0; i < (1 << 22); ++i) {
         uint32_t ok;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
@@ -439,9 +292,37 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int lim
             : "r"(bar), "r"(parity)
             : "memory");
         if (ok) return true;
-        __nanosleep(128);
+        if (i > 256) __nanosleep(128);
     }
     return false;
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {  // arrives when the MMAs issued so far are done
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
+                 : "memory");
+}
+
+// A bulk copy of `bytes` from global to shared memory that completes on `bar`.
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(bar)
+        : "memory");
+}
+
+// `steps` MMAs of K 16 of a 128-row A chunk (sbo 4096) and a 256-row B chunk into
+// the accumulator columns at `acc`; the first overwrites unless `add`.
+__device__ __forceinline__ void mma_chunk(uint32_t acc, uint32_t A, uint32_t B, uint32_t sbo, int steps, bool add) {
+    constexpr uint32_t idesc = umma_idesc_bf16_f32(kFwdRows, 256);
+    for (int ks = 0; ks < steps; ++ks)
+        asm volatile(
+            "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(acc),
+            "l"(umma_desc(A + uint32_t(ks) * 256, 128, 4096)), "l"(umma_desc(B + uint32_t(ks) * 256, 128, sbo)),
+            "r"(idesc), "r"(int(add) + ks));
 }
 
 // tcgen05.ld of 32 consecutive FP32 accumulator columns of this thread's
@@ -463,127 +344,494 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// X: M x K BF16 row-major (K a multiple of 16, K <= 256, rows 16-byte
-// aligned), W: 256 x K BF16 row-major, bias[256]; outputs row-major with 256
-// columns: EPI kBiasTanh writes Cf = tanh(Z) and Cb = bf16(Cf), kBiasLinear
-// Cf = Z. Grid (M / 128 rounded up, 2). `err` receives 1 if the accumulator
-// wait ran out (the tile's outputs are then not written).
-__device__ __forceinline__ void cp_async_wait_dyn(int n) {  // n in 0..3 groups may stay in flight
-    if (n <= 0) cp_async_wait<0>();
-    else if (n == 1) cp_async_wait<1>();
-    else if (n == 2) cp_async_wait<2>();
-    else cp_async_wait<3>();
-}
+// feat: n x 32 FP32; Wp: the operand images (packed_offset); p: the FP32
+// parameters (biases; L's offsets), W5: the output layer's BF16 weights 4 x 256.
+// out: n x 4. TRAIN: also Af[l], Ab[l] (n x 256) of the hidden layers, and Ab[0].
+// *err receives 1 if a wait ran out (the outputs are then incomplete).
+struct FwdStore {
+    float* Af[kLayers];
+    __nv_bfloat16* Ab[kLayers];
+};
 
-template <int EPI>
-__global__ void __launch_bounds__(kUmmaThreads, 1) k_gemm_fwd_umma(const __nv_bfloat16* __restrict__ X,
-                                                                   int M, int K,
-                                                                   const __nv_bfloat16* __restrict__ W,
-                                                                   const float* __restrict__ bias,
-                                                                   float* __restrict__ Cf,
-                                                                   __nv_bfloat16* __restrict__ Cb,
-                                                                   int* __restrict__ err) {
+template <bool TRAIN>
+__global__ void __launch_bounds__(kFwdThreads, 1)
+    k_forward(const float* __restrict__ feat, int64_t n, const unsigned char* __restrict__ Wp,
+              const float* __restrict__ p, LayerPtrs L, float* __restrict__ out, FwdStore st,
+              int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * kUmmaM, n0 = blockIdx.y * kUmmaN;
-    const uint32_t sA = smem_u32(smem);
-    const uint32_t sB = sA + uint32_t(kUmmaM * K * 2);
-    const uint32_t bar = sB + uint32_t(kUmmaN * K * 2);
-    const uint32_t tslot = bar + 8;
-    const uint32_t sbo = uint32_t(K) * 16;  // bytes between 8-row groups
-    const int kc = K / 8;                   // 16-byte chunks per row
-    const int nst = (K + kUmmaStageK - 1) / kUmmaStageK;  // 1..4 stages
+    const uint32_t sA = smem_u32(smem), sRing = sA + kFwdOffRing;
+    float* s_bias = reinterpret_cast<float*>(smem + kFwdOffBias);
+    float4* s_w5 = reinterpret_cast<float4*>(smem + kFwdOffW5);
+    float4* s_part = reinterpret_cast<float4*>(smem + kFwdOffPart);
+    // barriers: full[4], empty[4], chunk of A ready [4], accumulators ready, row
+    // parts ready; then the tensor-memory address
+    const uint32_t bar = sA + kFwdOffBar, full = bar, empty = bar + 32, a_ready = bar + 64,
+                   acc_ready = bar + 96, part_ready = bar + 104, tslot = bar + 112;
+    const int64_t tiles = (n + kFwdRows - 1) / kFwdRows;
 
-    // every stage's copies up front, one group per stage: chunk c of row r
-    // lands in core matrix (r/8, c)
-    for (int st = 0; st < nst; ++st) {
-        const int c0 = st * (kUmmaStageK / 8), c1 = min(kc, c0 + kUmmaStageK / 8), w = c1 - c0;
-        for (int i = tid; i < kUmmaM * w; i += kUmmaThreads) {
-            const int r = i / w, c = c0 + (i - r * w), gm = m0 + r;
-            const bool ok = gm < M;
-            cp_async16(sA + uint32_t(r >> 3) * sbo + uint32_t(c) * 128 + uint32_t(r & 7) * 16,
-                       ok ? X + int64_t(gm) * K + c * 8 : X, ok);
+    if (tid == 0) {
+        for (int i = 0; i < 4; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full + 8 * i));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(empty + 8 * i));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(a_ready + 8 * i), "r"(kFwdEpi));
         }
-        for (int i = tid; i < kUmmaN * w; i += kUmmaThreads) {
-            const int r = i / w, c = c0 + (i - r * w);
-            cp_async16(sB + uint32_t(r >> 3) * sbo + uint32_t(c) * 128 + uint32_t(r & 7) * 16,
-                       W + int64_t(n0 + r) * K + c * 8, true);
-        }
-        cp_async_commit();
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(acc_ready));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(part_ready), "r"(kFwdRows));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    if (warp == 0) {  // 128 columns x 128 lanes of 32-bit accumulators
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tslot),
-                     "r"(kUmmaN));
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(tslot));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar));
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    }
-    uint32_t tmem = 0;
-    constexpr uint32_t idesc = umma_idesc_bf16_f32(kUmmaM, kUmmaN);
-    for (int st = 0; st < nst; ++st) {
-        cp_async_wait_dyn(nst - 1 - st);  // this thread's copies of stages 0..st have landed
-        // the staged operands become visible to the tensor cores (async proxy)
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        __syncthreads();  // ... everyone's
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        if (st == 0) asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
-        if (tid == 0) {
-            const int k1 = min(K, (st + 1) * kUmmaStageK) / kUmmaK;
-            for (int ks = st * (kUmmaStageK / kUmmaK); ks < k1; ++ks) {
-                const uint64_t da = umma_desc(sA + uint32_t(ks) * 256, 128, sbo);
-                const uint64_t db = umma_desc(sB + uint32_t(ks) * 256, 128, sbo);
-                asm volatile(
-                    "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(da), "l"(db), "r"(idesc), "r"(ks));
-            }
-            if (st == nst - 1)
-                asm volatile(
-                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-                    : "memory");
-        }
-    }
-    // the accumulators are complete when the mbarrier's phase 0 completes
-    // (microseconds; the limit, ~0.5 s, only ends a wait that would not)
-    const bool done = __all_sync(0xffffffffu, mbar_wait(bar, 0, 1 << 22));
-    if (!done && lane == 0) atomicExch(err, 1);
+    for (int i = tid; i < kFwdHidden * 256; i += kFwdThreads) s_bias[i] = p[L.b_off[i >> 8] + (i & 255)];
+    for (int i = tid; i < 256; i += kFwdThreads)
+        s_w5[i] = make_float4(__bfloat162float(L.W[kLayers - 1][i]), __bfloat162float(L.W[kLayers - 1][256 + i]),
+                              __bfloat162float(L.W[kLayers - 1][512 + i]),
+                              __bfloat162float(L.W[kLayers - 1][768 + i]));
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (done) {
-        const int q = warp & 3, h = warp >> 2;
-        const int m = m0 + q * 32 + lane;  // this thread's row = its tensor-memory lane
-        for (int cc = 0; cc < kUmmaN / 2; cc += 32) {
-            const int c0 = h * (kUmmaN / 2) + cc;  // column within this CTA's half
-            float v[32];
-            tmem_ld32(tmem + (uint32_t(q * 32) << 16) + uint32_t(c0), v);
-            if (m < M) {
-                const int n = n0 + c0;
-                float4* of = reinterpret_cast<float4*>(Cf + int64_t(m) * kUmmaOut + n);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float4 o;
-                    o.x = v[4 * j] + __ldg(bias + n + 4 * j);
-                    o.y = v[4 * j + 1] + __ldg(bias + n + 4 * j + 1);
-                    o.z = v[4 * j + 2] + __ldg(bias + n + 4 * j + 2);
-                    o.w = v[4 * j + 3] + __ldg(bias + n + 4 * j + 3);
-                    if (EPI == kBiasTanh) {
-                        o.x = tanhf(o.x); o.y = tanhf(o.y); o.z = tanhf(o.z); o.w = tanhf(o.w);
-                        __nv_bfloat162* ob =
-                            reinterpret_cast<__nv_bfloat162*>(Cb + int64_t(m) * kUmmaOut + n + 4 * j);
-                        ob[0] = __floats2bfloat162_rn(o.x, o.y);
-                        ob[1] = __floats2bfloat162_rn(o.z, o.w);
-                    }
-                    of[j] = o;
+    uint32_t tmem;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
+    bool ok = true;
+
+    if (warp == 9) {  // weight copies
+        if (lane == 0) {
+            int64_t g = 0;  // chunk counter
+            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+                const unsigned char* src = Wp;
+                for (int c = 0; c < kFwdChunks; ++c, ++g) {
+                    const int slot = int(g % kFwdSlots);
+                    const uint32_t bytes = c == 0 ? kFwdIn0Bytes : kFwdSlotBytes;
+                    if (g >= kFwdSlots) ok = mbar_wait(empty + 8 * slot, uint32_t(g / kFwdSlots - 1) & 1u);
+                    if (!ok) break;
+                    bulk_copy(sRing + uint32_t(slot * kFwdSlotBytes), src, bytes, full + 8 * slot);
+                    src += bytes;
+                }
+            }
+            // no copy may be in flight when the CTA ends
+            for (int64_t i = max(int64_t(0), g - kFwdSlots); i < g; ++i)
+                ok = mbar_wait(full + 8 * int(i % kFwdSlots), uint32_t(i / kFwdSlots) & 1u) && ok;
+        }
+    } else if (warp == 8) {  // MMAs
+        if (lane == 0) {
+            int64_t g = 0, t = 0;
+            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
+                for (int c = 0; c < kFwdChunks && ok; ++c, ++g) {
+                    const int l = c == 0 ? 0 : (c + 3) / 4, kc = c == 0 ? 0 : (c - 1) % 4;
+                    const int slot = int(g % kFwdSlots);
+                    // the chunk of A: layer 0 fills only chunk 0
+                    const int64_t phase = kc == 0 ? t * kFwdHidden + l : t * (kFwdHidden - 1) + l - 1;
+                    ok = mbar_wait(a_ready + 8 * kc, uint32_t(phase) & 1u) &&
+                         mbar_wait(full + 8 * slot, uint32_t(g / kFwdSlots) & 1u);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    mma_chunk(tmem + uint32_t(l & 1) * 256, sA + uint32_t(kc * 1024),
+                              sRing + uint32_t(slot * kFwdSlotBytes), c == 0 ? 512u : 1024u, c == 0 ? 2 : 4,
+                              kc > 0);
+                    mma_commit(empty + 8 * slot);
+                    if (c == 0 || kc == 3) mma_commit(acc_ready);
                 }
             }
         }
+    } else {  // epilogue
+        const int quarter = warp & 3, half = warp >> 2;
+        const int row = quarter * 32 + lane;  // of the tile; this thread's tensor-memory lane
+        int64_t t = 0;
+        for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
+            const int64_t m = tile * kFwdRows + row;
+            const bool live = m < n;
+            {   // the features as BF16: half a row a thread
+                uint32_t v[8];
+                const float4* f = reinterpret_cast<const float4*>(feat + m * kIn + half * 16);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 x = live ? f[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
+                    v[2 * i] = *reinterpret_cast<const uint32_t*>(&a);
+                    v[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&b);
+                }
+                unsigned char* dst = smem + (row >> 3) * 4096 + half * 256 + (row & 7) * 16;
+                *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<uint4*>(dst + 128) = make_uint4(v[4], v[5], v[6], v[7]);
+                if (TRAIN && live) {
+                    uint4* o = reinterpret_cast<uint4*>(st.Ab[0] + m * kIn + half * 16);
+                    o[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                    o[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                mbar_arrive(a_ready);
+            }
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int l = 0; l < kFwdHidden; ++l) {
+                ok = __all_sync(0xffffffffu, mbar_wait(acc_ready, uint32_t(t * kFwdHidden + l) & 1u));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const float* bias = s_bias + l * 256;
+                for (int kc = 0; kc < 4; ++kc) {  // 64 columns: the next layer's chunk of k
+                    const int c0 = kc * 64 + half * 32;
+                    float v[32];
+                    tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t((l & 1) * 256 + c0), v);
+                    uint32_t b[16];
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 bj = *reinterpret_cast<const float4*>(bias + c0 + j);
+                        v[j] = tanhf(v[j] + bj.x);
+                        v[j + 1] = tanhf(v[j + 1] + bj.y);
+                        v[j + 2] = tanhf(v[j + 2] + bj.z);
+                        v[j + 3] = tanhf(v[j + 3] + bj.w);
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[j], v[j + 1]),
+                                             hi = __floats2bfloat162_rn(v[j + 2], v[j + 3]);
+                        b[j / 2] = *reinterpret_cast<const uint32_t*>(&lo);
+                        b[j / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+                    }
+                    if (l < kFwdHidden - 1) {
+                        unsigned char* dst = smem + (row >> 3) * 4096 + (c0 >> 3) * 128 + (row & 7) * 16;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            *reinterpret_cast<uint4*>(dst + j * 128) =
+                                make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                        mbar_arrive(a_ready + 8 * kc);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const uint32_t w = b[j / 2];
+                            const float x = __uint_as_float(j & 1 ? w & 0xffff0000u : w << 16);
+                            const float4 w5 = s_w5[c0 + j];
+                            y.x = fmaf(x, w5.x, y.x);
+                            y.y = fmaf(x, w5.y, y.y);
+                            y.z = fmaf(x, w5.z, y.z);
+                            y.w = fmaf(x, w5.w, y.w);
+                        }
+                    }
+                    if (TRAIN && live) {
+                        float4* of = reinterpret_cast<float4*>(st.Af[l + 1] + m * kWidth + c0);
+                        uint4* ob = reinterpret_cast<uint4*>(st.Ab[l + 1] + m * kWidth + c0);
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) of[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            ob[j] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                    }
+                }
+            }
+            if (!ok) break;
+            // the two column halves of a row (a thread of the second half writes its
+            // next part only after every thread has passed the next tile's layers)
+            if (half == 1) {
+                s_part[row] = y;
+                mbar_arrive(part_ready);
+                continue;
+            }
+            ok = __all_sync(0xffffffffu, mbar_wait(part_ready, uint32_t(t) & 1u));
+            if (ok && live) {
+                const float4 z = s_part[row];
+                const float* b5 = p + L.b_off[kLayers - 1];
+                reinterpret_cast<float4*>(out)[m] = make_float4(y.x + z.x + b5[0], y.y + z.y + b5[1],
+                                                                y.z + z.z + b5[2], y.w + z.w + b5[3]);
+            }
+        }
     }
+    if (!ok && lane == 0) *err = 1;
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kUmmaN));
+    __syncwarp();
+    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+// ------------------------------------------------- fused backward pass
+// The error signals of a 128-row tile from the output to the first layer in one
+// CTA, as k_forward runs forwards (8,192 samples: loss and gradients 659 us with
+// a launch for each layer's product, sum and tanh', now 204): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
+// dZ_(l-1) = (dZ_l W_l) (1 - A_l^2) for l = 4..1 with the products on the tensor
+// cores. Stores each layer's dZ in BF16 (the weight gradients' operand), the
+// column sums of the FP32 dZ (the bias gradients; one row of partial sums for
+// each CTA and tensor-memory quarter) and the squared error.
+constexpr int kBwdSums = kFwdHidden * kWidth;  // columns of a partial row; then dY's 4
+
+struct BwdArgs {
+    const float* Y;  // n x 4 outputs and targets
+    const float* T;
+    const float* Af[kLayers];      // A_l, l = 1..5
+    __nv_bfloat16* dZb[kLayers];   // dZ_l, l = 0..4 (n x 256), 5 (n x 4)
+    const unsigned char* Wt;       // transposed operand images
+    const __nv_bfloat16* W5;       // 4 x 256
+    float* sums;                   // [4 gridDim][kBwdSums + 4]
+    double* sq;                    // [4 gridDim]
+};
+
+__global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, int64_t n, int* __restrict__ err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t sA = smem_u32(smem), sRing = sA + kFwdOffRing;
+    float4* s_w5 = reinterpret_cast<float4*>(smem + kFwdOffW5);
+    const uint32_t bar = sA + kFwdOffBar, full = bar, empty = bar + 32, a_ready = bar + 64,
+                   acc_ready = bar + 96, tslot = bar + 112;
+    const int64_t tiles = (n + kFwdRows - 1) / kFwdRows;
+    constexpr int kSteps = kFwdHidden - 1;  // layers on the tensor cores
+
+    if (tid == 0) {
+        for (int i = 0; i < 4; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full + 8 * i));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(empty + 8 * i));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(a_ready + 8 * i), "r"(kFwdEpi));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(acc_ready));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(tslot));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+    }
+    for (int i = tid; i < 256; i += kFwdThreads)
+        s_w5[i] = make_float4(__bfloat162float(a.W5[i]), __bfloat162float(a.W5[256 + i]),
+                              __bfloat162float(a.W5[512 + i]), __bfloat162float(a.W5[768 + i]));
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    uint32_t tmem;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
+    bool ok = true;
+
+    if (warp == 9) {  // weight copies
+        if (lane == 0) {
+            int64_t g = 0;
+            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+                const unsigned char* src = a.Wt;
+                for (int c = 0; c < 4 * kSteps; ++c, ++g, src += kFwdSlotBytes) {
+                    const int slot = int(g % kFwdSlots);
+                    if (g >= kFwdSlots) ok = mbar_wait(empty + 8 * slot, uint32_t(g / kFwdSlots - 1) & 1u);
+                    if (!ok) break;
+                    bulk_copy(sRing + uint32_t(slot * kFwdSlotBytes), src, kFwdSlotBytes, full + 8 * slot);
+                }
+            }
+            for (int64_t i = max(int64_t(0), g - kFwdSlots); i < g; ++i)
+                ok = mbar_wait(full + 8 * int(i % kFwdSlots), uint32_t(i / kFwdSlots) & 1u) && ok;
+        }
+    } else if (warp == 8) {  // MMAs
+        if (lane == 0) {
+            int64_t g = 0;
+            for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+                for (int c = 0; c < 4 * kSteps && ok; ++c, ++g) {
+                    const int kc = c % 4, slot = int(g % kFwdSlots);
+                    ok = mbar_wait(a_ready + 8 * kc, uint32_t(g / 4) & 1u) &&
+                         mbar_wait(full + 8 * slot, uint32_t(g / kFwdSlots) & 1u);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    mma_chunk(tmem + uint32_t(c / 4 & 1) * 256, sA + uint32_t(kc * 1024),
+                              sRing + uint32_t(slot * kFwdSlotBytes), 1024, 4, kc > 0);
+                    mma_commit(empty + 8 * slot);
+                    if (kc == 3) mma_commit(acc_ready);
+                }
+            }
+        }
+    } else {  // epilogue
+        const int quarter = warp & 3, half = warp >> 2;
+        const int row = quarter * 32 + lane;
+        const float scale = float(n * kOut);
+        float db[kFwdHidden][4] = {};  // this lane's columns: layer, chunk
+        float4 db5 = make_float4(0.f, 0.f, 0.f, 0.f);
+        double sq = 0.0;
+        int64_t t = 0;
+        for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
+            const int64_t m = tile * kFwdRows + row;
+            const bool live = m < n;
+            // dY = 2 (Y - T) / (4 n), and its BF16 rounding
+            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (live) {
+                const float* y = a.Y + m * kOut;
+                const float* g = a.T + m * kOut;
+                d = make_float4(y[0] - g[0], y[1] - g[1], y[2] - g[2], y[3] - g[3]);
+            }
+            const float4 dy = make_float4(2.0f * d.x / scale, 2.0f * d.y / scale, 2.0f * d.z / scale,
+                                          2.0f * d.w / scale);
+            const __nv_bfloat162 b01 = __floats2bfloat162_rn(dy.x, dy.y), b23 = __floats2bfloat162_rn(dy.z, dy.w);
+            const float2 r01 = __bfloat1622float2(b01), r23 = __bfloat1622float2(b23);
+            if (half == 0) {
+                sq += double(d.x) * d.x + double(d.y) * d.y + double(d.z) * d.z + double(d.w) * d.w;
+                db5.x += dy.x;
+                db5.y += dy.y;
+                db5.z += dy.z;
+                db5.w += dy.w;
+                if (live)
+                    reinterpret_cast<uint2*>(a.dZb[kLayers - 1])[m] =
+                        make_uint2(*reinterpret_cast<const uint32_t*>(&b01), *reinterpret_cast<const uint32_t*>(&b23));
+            }
+#pragma unroll
+            for (int i = 0; i < kFwdHidden; ++i) {  // dZ_l, l = 4 - i
+                const int l = kFwdHidden - 1 - i;
+                if (i > 0) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(acc_ready, uint32_t(t * kSteps + i - 1) & 1u));
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                }
+                const float* act = a.Af[l + 1] + m * kWidth;
+                __nv_bfloat16* to = a.dZb[l] + m * kWidth;
+#pragma unroll
+                for (int kc = 0; kc < 4; ++kc) {
+                    const int c0 = kc * 64 + half * 32;
+                    float v[32];
+                    if (i == 0) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float4 w = s_w5[c0 + j];
+                            v[j] = fmaf(r23.y, w.w, fmaf(r23.x, w.z, fmaf(r01.y, w.y, r01.x * w.x)));
+                        }
+                    } else {
+                        tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(((i - 1) & 1) * 256 + c0), v);
+                    }
+                    uint32_t b[16];
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 x = live ? *reinterpret_cast<const float4*>(act + c0 + j)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                        v[j] *= 1.0f - x.x * x.x;
+                        v[j + 1] *= 1.0f - x.y * x.y;
+                        v[j + 2] *= 1.0f - x.z * x.z;
+                        v[j + 3] *= 1.0f - x.w * x.w;
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[j], v[j + 1]),
+                                             hi = __floats2bfloat162_rn(v[j + 2], v[j + 3]);
+                        b[j / 2] = *reinterpret_cast<const uint32_t*>(&lo);
+                        b[j / 2 + 1] = *reinterpret_cast<const uint32_t*>(&hi);
+                    }
+                    if (l > 0) {
+                        unsigned char* dst = smem + (row >> 3) * 4096 + (c0 >> 3) * 128 + (row & 7) * 16;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            *reinterpret_cast<uint4*>(dst + j * 128) =
+                                make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                        mbar_arrive(a_ready + 8 * kc);
+                    }
+                    if (live) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            reinterpret_cast<uint4*>(to + c0)[j] =
+                                make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                    }
+                    // the 32 rows' sums of 32 columns: lane j ends with column j
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                        for (int j = 0; j < o; ++j) {
+                            const float keep = lane & o ? v[j + o] : v[j], give = lane & o ? v[j] : v[j + o];
+                            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                        }
+                    db[l][kc] += v[0];
+                }
+            }
+        }
+        // partial sums: one row for each CTA and quarter
+        const int64_t r = int64_t(blockIdx.x) * 4 + quarter;
+        float* out = a.sums + r * (kBwdSums + kOut);
+#pragma unroll
+        for (int l = 0; l < kFwdHidden; ++l)
+#pragma unroll
+            for (int kc = 0; kc < 4; ++kc) out[l * kWidth + kc * 64 + half * 32 + lane] = db[l][kc];
+        if (half == 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                db5.x += __shfl_xor_sync(0xffffffffu, db5.x, o);
+                db5.y += __shfl_xor_sync(0xffffffffu, db5.y, o);
+                db5.z += __shfl_xor_sync(0xffffffffu, db5.z, o);
+                db5.w += __shfl_xor_sync(0xffffffffu, db5.w, o);
+            }
+            if (lane == 0) {
+                a.sq[r] = sq;
+                out[kBwdSums] = db5.x;
+                out[kBwdSums + 1] = db5.y;
+                out[kBwdSums + 2] = db5.z;
+                out[kBwdSums + 3] = db5.w;
+            }
+        }
+    }
+    if (!ok && lane == 0) *err = 1;
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    __syncwarp();
+    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+}
+
+// All weight gradients of a slice of the samples, dW_l = dZ_l^T X_l, in one launch:
+// blockIdx.y 0..3 the layers 1..4 (four 128 x 128 tiles), 4 the first layer (two
+// 128 x 32 ones), 5 the output layer. Slice z goes to part + z * np, a whole
+// parameter vector.
+struct DwArgs {
+    const __nv_bfloat16* dZb[kLayers];
+    const __nv_bfloat16* X[kLayers];
+    LayerPtrs L;
+    float* part;
+    int64_t np;
+};
+
+__global__ void __launch_bounds__(256) k_weight_grads(const DwArgs a, int n, int kchunk) {
+    const int l = blockIdx.y < 4 ? blockIdx.y + 1 : blockIdx.y == 4 ? 0 : kLayers - 1;
+    const int kbeg = blockIdx.z * kchunk, kend = min(n, kbeg + kchunk);
+    float* part = a.part + int64_t(blockIdx.z) * a.np + a.L.w_off[l];
+    if (l == kLayers - 1) {  // 4 x 256: a thread a column, a quarter of the slice a block
+        const int q = (kend - kbeg + 3) / 4, s0 = kbeg + int(blockIdx.x) * q, s1 = min(kend, s0 + q);
+        float acc[kOut] = {0.f, 0.f, 0.f, 0.f};
+        const __nv_bfloat16* x = a.X[l] + threadIdx.x;
+        const uint2* dz = reinterpret_cast<const uint2*>(a.dZb[l]);
+#pragma unroll 4
+        for (int s = s0; s < s1; ++s) {
+            const float xv = __bfloat162float(x[int64_t(s) * kWidth]);
+            const uint2 d = dz[s];
+            acc[0] = fmaf(xv, __uint_as_float(d.x << 16), acc[0]);
+            acc[1] = fmaf(xv, __uint_as_float(d.x & 0xffff0000u), acc[1]);
+            acc[2] = fmaf(xv, __uint_as_float(d.y << 16), acc[2]);
+            acc[3] = fmaf(xv, __uint_as_float(d.y & 0xffff0000u), acc[3]);
+        }
+        // the quarters' rows go after the vectors of the slices
+        float* to = a.part + int64_t(gridDim.z) * a.np + (int64_t(blockIdx.z) * 4 + blockIdx.x) * (kOut * kWidth);
+        for (int o = 0; o < kOut; ++o) to[o * kWidth + threadIdx.x] = acc[o];
+        return;
+    }
+    if (l == 0 && blockIdx.x >= 2) return;
+    const int K = layer_in(l);
+    gemm_tc_block<false, false>(a.dZb[l], 1, kWidth, a.X[l], K, 1, kWidth, K, kbeg, kend,
+                                l == 0 ? int(blockIdx.x) * kTB : int(blockIdx.x >> 1) * kTB,
+                                l == 0 ? 0 : int(blockIdx.x & 1) * kTB, part, K);
+}
+
+// The gradient vector from the slices (in slice order) and the partial column
+// sums, and the loss: mean squared error.
+__global__ void __launch_bounds__(256) k_reduce_grads(const DwArgs a, int slices, const float* __restrict__ sums,
+                                                      const double* __restrict__ sq, int rows, double count,
+                                                      float* __restrict__ g, double* __restrict__ loss) {
+    const int64_t e = int64_t(blockIdx.x) * 256 + threadIdx.x;
+    if (e == 0) {
+        double s = 0.0;
+        for (int r = 0; r < rows; ++r) s += sq[r];
+        *loss = s / count;
+    }
+    if (e >= a.np) return;
+    int l = kLayers - 1;
+    while (e < a.L.w_off[l]) --l;
+    float s = 0.f;
+    if (e < a.L.b_off[l]) {
+        if (l < kLayers - 1) {
+#pragma unroll 4
+            for (int z = 0; z < slices; ++z) s += a.part[int64_t(z) * a.np + e];
+        } else {
+            const float* p = a.part + int64_t(slices) * a.np + (e - a.L.w_off[l]);
+#pragma unroll 4
+            for (int z = 0; z < 4 * slices; ++z) s += p[int64_t(z) * (kOut * kWidth)];
+        }
+    } else {
+        const float* p = sums + (l < kLayers - 1 ? l * kWidth : kBwdSums) + (e - a.L.b_off[l]);
+#pragma unroll 8
+        for (int r = 0; r < rows; ++r) s += p[int64_t(r) * (kBwdSums + kOut)];
+    }
+    g[e] = s;
 }
 
 // Features: per sample raw (x, y, wall distance, M, alpha_deg) ->
@@ -612,85 +860,7 @@ __global__ void k_features(const float* __restrict__ raw, int64_t n, const float
     for (int k = 21; k < kIn; ++k) f[k] = 0.f;
 }
 
-// Sum of the split-K slices in slice order (deterministic).
-__global__ void k_sum_slices(const float* __restrict__ part, int slices, int64_t n,
-                             float* __restrict__ out) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-    for (int z = 0; z < slices; ++z) s += part[int64_t(z) * n + i];
-    out[i] = s;
-}
-
-__global__ void k_to_bf16(const float* __restrict__ src, int64_t n, __nv_bfloat16* __restrict__ dst) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = __float2bfloat16(src[i]);
-}
-
-// MSE loss pieces: dY = 2 (Y - T) / (n * 4), per-block partial sums of (Y-T)^2.
-__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ Y, const float* __restrict__ T,
-                                             int64_t n, float* __restrict__ dY,
-                                             double* __restrict__ partial) {
-    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    double s = 0.0;
-    if (i < n * kOut) {
-        const float d = Y[i] - T[i];
-        dY[i] = 2.0f * d / float(n * kOut);
-        s = double(d) * d;
-    }
-    __shared__ double sh[256];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-__global__ void k_sum_partials(const double* __restrict__ partial, int nb, int64_t count,
-                               double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += partial[b];
-    *out = s / double(count);
-}
-
-// dZ = dA * (1 - A^2) (tanh'), FP32 and BF16 copies.
-__global__ void k_tanh_back(const float* __restrict__ dA, const float* __restrict__ A, int64_t n,
-                            float* __restrict__ dZ, __nv_bfloat16* __restrict__ dZb) {
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float a = A[i];
-    const float v = dA[i] * (1.0f - a * a);
-    dZ[i] = v;
-    dZb[i] = __float2bfloat16(v);
-}
-
-// db[c] = sum over rows of dZ[r][c], rows summed in a fixed order.
-__global__ void __launch_bounds__(256) k_colsum(const float* __restrict__ dZ, int rows, int cols,
-                                                float* __restrict__ db) {
-    __shared__ float sh[8][33];
-    const int c = blockIdx.x * 32 + threadIdx.x;
-    float s = 0.f;
-    if (c < cols)
-        for (int r = threadIdx.y; r < rows; r += 8) s += dZ[int64_t(r) * cols + c];
-    sh[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0 && c < cols) {
-        float t = 0.f;
-        for (int k = 0; k < 8; ++k) t += sh[k][threadIdx.x];
-        db[c] = t;
-    }
-}
-
-// Adam on the flat FP32 parameter vector; the BF16 copy W is refreshed after it.
-struct LayerPtrs {
-    int64_t w_off[kLayers];  // offsets of W_l and b_l in the flat vector
-    int64_t b_off[kLayers];
-    __nv_bfloat16* W[kLayers];
-};
-
+// Adam on the flat FP32 parameter vector; the BF16 copies are refreshed after it.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
                        float c1, float c2) {
@@ -704,16 +874,21 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
 }
 
-__global__ void k_weights_bf16(const float* __restrict__ p, LayerPtrs L) {
+// BF16 copies of the weights: row-major, and as the operand images of the fused
+// forward and backward passes.
+__global__ void k_weights_bf16(const float* __restrict__ p, LayerPtrs L, unsigned char* __restrict__ Wp,
+                               unsigned char* __restrict__ Wt) {
     const int l = blockIdx.y;
     const int K = layer_in(l), N = layer_out(l);
     const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (e >= int64_t(K) * N) return;
-    const int nrow = int(e / K), k = int(e % K);
+    const int row = int(e / K), k = int(e % K);
     float w = p[L.w_off[l] + e];
     if (l == 0 && k >= 21) w = 0.f;  // padded inputs carry no weight
-    L.W[l][e] = __float2bfloat16(w);
-    (void)nrow;
+    const __nv_bfloat16 b = __float2bfloat16(w);
+    L.W[l][e] = b;
+    if (l < kLayers - 1) *reinterpret_cast<__nv_bfloat16*>(Wp + packed_offset(l, row, k)) = b;
+    if (l > 0 && l < kLayers - 1) *reinterpret_cast<__nv_bfloat16*>(Wt + packed_offset_t(l, row, k)) = b;
 }
 
 }  // namespace mlpk
@@ -737,14 +912,15 @@ struct lskum_mlp {
     // activations: Af[l] (FP32) and Ab[l] (BF16) for l = 0..kLayers (l = 0: features)
     float* Af[kLayers + 1] = {nullptr};
     __nv_bfloat16* Ab[kLayers + 1] = {nullptr};
-    float* dA = nullptr;   // cap x 256 scratch
-    float* slices = nullptr;  // split-K partial products of the weight gradients
-    float* dZ = nullptr;   // cap x 256
-    __nv_bfloat16* dZb = nullptr;
-    double* partial = nullptr;
+    __nv_bfloat16* dZb[kLayers] = {nullptr};  // error signals (BF16)
+    float* slices = nullptr;  // partial weight gradients: a parameter vector for each slice
+    float* sums = nullptr;    // partial bias gradients: a row for each CTA and quarter
+    double* partial = nullptr;  // and squared errors
     double* loss_dev = nullptr;
-    int gemm_path = LSKUM_MLP_GEMM_MMA_SYNC;
-    int* err_dev = nullptr;  // set by a tcgen05 GEMM whose accumulator wait ran out
+    unsigned char* Wp = nullptr;  // operand images of the weights: forward pass
+    unsigned char* Wt = nullptr;  // and backward pass
+    int sms = 0;
+    int* err = nullptr;  // pinned: set by a forward pass one of whose waits ran out
     std::vector<void*> allocs;
 };
 
@@ -773,170 +949,82 @@ cudaError_t alloc(lskum_mlp* h, T** p, int64_t count) {
 
 inline unsigned blocks(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
-constexpr int kMaxSlices = 32;
-
-// The pipelined kernel's layout requirements (see k_gemm_bf16_tc); small
-// outputs (the 4-wide output layer, the 32-wide input layer's weight
-// gradient) stay on the 64 x 64 kernel.
-bool tc_ok(const void* A, int64_t sam, int64_t sak, const void* B, int64_t sbk, int64_t sbn, int M,
-           int N, int K) {
-    if (M < 64 || N < 64) return false;
-    const bool ak = sak == 1, bk = sbk == 1;
-    if ((!ak && sam != 1) || (!bk && sbn != 1)) return false;
-    if ((reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(B) & 15)) return false;
-    if (ak ? (sam % 8 || K % 8) : (sak % 8 || M % 8)) return false;
-    if (bk ? (sbn % 8 || K % 8) : (sbk % 8 || N % 8)) return false;
-    return true;
-}
-
-template <int EPI, bool AK, bool BK>
-cudaError_t launch_tc(lskum_mlp* h, dim3 grid, const __nv_bfloat16* A, int64_t sam, int64_t sak,
-                      const __nv_bfloat16* B, int64_t sbk, int64_t sbn, int M, int N, int K,
-                      const float* bias, float* Cf, __nv_bfloat16* Cb, int64_t ldc, int kchunk) {
-    constexpr size_t smem = tc_smem_bytes(AK, BK);
-    // the opt-in above 48 KB of dynamic shared memory (per device, so set on
-    // every launch: a cheap host call next to a GEMM)
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_bf16_tc<EPI, AK, BK>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    k_gemm_bf16_tc<EPI, AK, BK><<<grid, 256, smem, h->stream>>>(A, sam, sak, B, sbk, sbn, M, N, K, bias,
-                                                                Cf, Cb, ldc, kchunk);
-    return cudaGetLastError();
-}
-
-// The tcgen05 forward GEMM's requirements: 256 outputs, K a multiple of 16 up
-// to 256 (16-byte rows), 16-byte aligned operands.
-bool umma_ok(const void* X, const void* W, int N, int K) {
-    return N == kUmmaOut && K % kUmmaK == 0 && K >= kUmmaK && K <= 256 &&
-           !(reinterpret_cast<uintptr_t>(X) & 15) && !(reinterpret_cast<uintptr_t>(W) & 15);
-}
-
-template <int EPI>
-cudaError_t launch_umma(lskum_mlp* h, const __nv_bfloat16* X, int M, int K, const __nv_bfloat16* W,
-                        const float* bias, float* Cf, __nv_bfloat16* Cb) {
-    // at least 60 KB, so at most three CTAs share an SM: their 128-column
-    // accumulators fit its 512 tensor-memory columns and no allocation waits
-    const size_t smem = std::max<size_t>(umma_smem_bytes(K), 60 * 1024);
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_fwd_umma<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(umma_smem_bytes(256)));
-    if (e != cudaSuccess) return e;
-    const dim3 grid(blocks(M, kUmmaM), kUmmaOut / kUmmaN);
-    k_gemm_fwd_umma<EPI><<<grid, kUmmaThreads, smem, h->stream>>>(X, M, K, W, bias, Cf, Cb, h->err_dev);
-    return cudaGetLastError();
-}
+constexpr int kMaxSlices = 16;
+constexpr int kDwSmem = int(tc_smem_bytes(false, false));
 
 // After a synchronising call: LSKUM_ERR_TIMEOUT (and the flag cleared) if a
-// tcgen05 GEMM gave up waiting for its accumulators.
+// forward pass gave up one of its waits.
 int check_gemm_status(lskum_mlp* h) {
-    if (h->gemm_path != LSKUM_MLP_GEMM_TCGEN05) return LSKUM_OK;
-    int flag = 0;
-    MLP_CUDA(cudaMemcpy(&flag, h->err_dev, sizeof(int), cudaMemcpyDeviceToHost));
-    if (!flag) return LSKUM_OK;
-    MLP_CUDA(cudaMemset(h->err_dev, 0, sizeof(int)));
-    return fail(LSKUM_ERR_TIMEOUT, "tcgen05 GEMM: accumulator wait ran out");
+    if (!*static_cast<volatile int*>(h->err)) return LSKUM_OK;
+    *h->err = 0;
+    return fail(LSKUM_ERR_TIMEOUT, "forward pass: a wait ran out");
 }
 
-template <int EPI>
-cudaError_t gemm(lskum_mlp* h, const __nv_bfloat16* A, int64_t sam, int64_t sak,
-                 const __nv_bfloat16* B, int64_t sbk, int64_t sbn, int M, int N, int K,
-                 const float* bias, float* Cf, __nv_bfloat16* Cb, int64_t ldc) {
-    // forward X W^T into few outputs (the last layer): a warp per row
-    if (EPI == kBiasLinear && sak == 1 && sbk == 1 && sbn == K && N <= kNarrowMax &&
-        int64_t(N) * K <= kNarrowW && K % 8 == 0 && sam % 8 == 0 &&
-        !(reinterpret_cast<uintptr_t>(A) & 15) && !(reinterpret_cast<uintptr_t>(B) & 15)) {
-        k_gemm_narrow<<<blocks(M, kNarrowRows), 32 * kNarrowRows, 0, h->stream>>>(A, sam, B, M, N, K,
-                                                                                  bias, Cf, ldc);
-        return cudaGetLastError();
-    }
-    if (tc_ok(A, sam, sak, B, sbk, sbn, M, N, K)) {
-        const dim3 grid(blocks(N, kTB), blocks(M, kTB), 1);
-        const int kchunk = int(blocks(K, kTK)) * kTK;
-        if (sak == 1 && sbk == 1)  // forward X W^T
-            return launch_tc<EPI, true, true>(h, grid, A, sam, sak, B, sbk, sbn, M, N, K, bias, Cf, Cb,
-                                              ldc, kchunk);
-        if (EPI == kStoreF32 && sak == 1)  // backward dZ W
-            return launch_tc<kStoreF32, true, false>(h, grid, A, sam, sak, B, sbk, sbn, M, N, K,
-                                                     nullptr, Cf, nullptr, ldc, kchunk);
-    }
-    dim3 grid(blocks(N, kTile), blocks(M, kTile), 1);
-    k_gemm_bf16<EPI><<<grid, 128, 0, h->stream>>>(A, sam, sak, B, sbk, sbn, M, N, K, bias, Cf, Cb, ldc,
-                                                   K);
-    return cudaGetLastError();
-}
-
-// C[M x N] (ldc = N) = A B with the contraction split over enough slices to
-// give ~4 blocks per SM: for the weight gradients, whose M x N is one 256 x
-// 256 tile grid while K is the batch.
-cudaError_t gemm_splitk(lskum_mlp* h, const __nv_bfloat16* A, int64_t sam, int64_t sak,
-                        const __nv_bfloat16* B, int64_t sbk, int64_t sbn, int M, int N, int K,
-                        float* C) {
-    const bool tc = tc_ok(A, sam, sak, B, sbk, sbn, M, N, K) && sam == 1 && sbn == 1;
-    const int tile = tc ? kTB : kTile;
-    const int tiles = int(blocks(N, tile) * blocks(M, tile));
-    int slices = std::min(kMaxSlices, std::max(1, (tc ? 300 : 600) / tiles));
-    int kchunk = int(blocks(K, slices));
-    kchunk = (kchunk + kKt - 1) / kKt * kKt;  // kKt == kTK: whole k stages per slice
-    slices = int(blocks(K, kchunk));
-    dim3 grid(blocks(N, tile), blocks(M, tile), slices);
-    cudaError_t e;
-    if (tc) {
-        // weight gradient dZ^T X: both operands transposed on load
-        e = launch_tc<kStoreF32, false, false>(h, grid, A, sam, sak, B, sbk, sbn, M, N, K, nullptr,
-                                               h->slices, nullptr, N, kchunk);
-    } else {
-        k_gemm_bf16<kStoreF32><<<grid, 128, 0, h->stream>>>(A, sam, sak, B, sbk, sbn, M, N, K, nullptr,
-                                                            h->slices, nullptr, N, kchunk);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) return e;
-    const int64_t n = int64_t(M) * N;
-    k_sum_slices<<<blocks(n, 256), 256, 0, h->stream>>>(h->slices, slices, n, C);
-    return cudaGetLastError();
-}
-
-// forward from features (FP32 n x 32 in h->Af[0]); output Af[kLayers] (n x 4)
-int forward(lskum_mlp* h, int64_t n) {
-    MLP_CUDA((k_to_bf16<<<blocks(n * kIn, 256), 256, 0, h->stream>>>(h->Af[0], n * kIn, h->Ab[0]),
-              cudaGetLastError()));
+// Forward pass from features (FP32 n x 32) to out (n x 4); train: the hidden
+// activations are kept for the backward pass.
+int forward(lskum_mlp* h, const float* feat, int64_t n, float* out, bool train) {
+    const int64_t tiles = (n + kFwdRows - 1) / kFwdRows;
+    const unsigned grid = unsigned(std::min<int64_t>(tiles, h->sms));
+    FwdStore st;
     for (int l = 0; l < kLayers; ++l) {
-        const int K = layer_in(l), N = layer_out(l);
-        const float* b = h->p + h->L.b_off[l];
-        cudaError_t e;
-        if (l < kLayers - 1 && h->gemm_path == LSKUM_MLP_GEMM_TCGEN05 && umma_ok(h->Ab[l], h->L.W[l], N, K))
-            e = launch_umma<kBiasTanh>(h, h->Ab[l], int(n), K, h->L.W[l], b, h->Af[l + 1], h->Ab[l + 1]);
-        else if (l < kLayers - 1)
-            e = gemm<kBiasTanh>(h, h->Ab[l], K, 1, h->L.W[l], 1, K, int(n), N, K, b, h->Af[l + 1],
-                                h->Ab[l + 1], N);
-        else
-            e = gemm<kBiasLinear>(h, h->Ab[l], K, 1, h->L.W[l], 1, K, int(n), N, K, b, h->Af[l + 1],
-                                  nullptr, N);
-        if (e != cudaSuccess) return fail(LSKUM_ERR_CUDA, std::string("forward: ") + cudaGetErrorString(e));
+        st.Af[l] = h->Af[l];
+        st.Ab[l] = h->Ab[l];
     }
+    if (train)
+        k_forward<true><<<grid, kFwdThreads, kFwdSmem, h->stream>>>(feat, n, h->Wp, h->p, h->L, out, st, h->err);
+    else
+        k_forward<false><<<grid, kFwdThreads, kFwdSmem, h->stream>>>(feat, n, h->Wp, h->p, h->L, out, st, h->err);
+    MLP_CUDA(cudaGetLastError());
     return LSKUM_OK;
+}
+
+// The features where the forward pass can read them with 16-byte loads while
+// `out` is written: the caller's, or a copy of them.
+int stage_features(lskum_mlp* h, const float* feat, int64_t n, const float* out, const float** use) {
+    const uintptr_t f = reinterpret_cast<uintptr_t>(feat), o = reinterpret_cast<uintptr_t>(out);
+    const bool apart = !out || o >= f + sizeof(float) * n * kIn || f >= o + sizeof(float) * n * kOut;
+    *use = feat;
+    if (!(f & 15) && apart) return LSKUM_OK;
+    MLP_CUDA(cudaMemcpyAsync(h->Af[0], feat, sizeof(float) * n * kIn, cudaMemcpyDeviceToDevice, h->stream));
+    *use = h->Af[0];
+    return LSKUM_OK;
+}
+
+// Slices of the weight gradients' contraction over n samples: at most
+// kMaxSlices of at least 256 samples, whole k stages each.
+int grad_kchunk(int64_t n) {
+    return int(std::max<int64_t>(256, ((n + kMaxSlices - 1) / kMaxSlices + kTK - 1) / kTK * kTK));
 }
 
 // backward from targets T (device n x 4): gradients into h->g, loss into loss_dev
 int backward(lskum_mlp* h, const float* T, int64_t n) {
-    const int nb = int(blocks(n * kOut, 256));
-    MLP_CUDA((k_mse<<<nb, 256, 0, h->stream>>>(h->Af[kLayers], T, n, h->dZ, h->partial), cudaGetLastError()));
-    MLP_CUDA((k_sum_partials<<<1, 32, 0, h->stream>>>(h->partial, nb, n * kOut, h->loss_dev), cudaGetLastError()));
-    // output layer: dZ (n x 4) FP32 in h->dZ
-    MLP_CUDA((k_to_bf16<<<blocks(n * kOut, 256), 256, 0, h->stream>>>(h->dZ, n * kOut, h->dZb), cudaGetLastError()));
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int K = layer_in(l), N = layer_out(l);
-        // dW_l [N x K] = dZ^T X_l : A(m = out unit, k = sample) = dZ[s][m], B(k = sample, n = in) = X[s][n]
-        cudaError_t e = gemm_splitk(h, h->dZb, 1, N, h->Ab[l], K, 1, N, K, int(n),
-                                    h->g + h->L.w_off[l]);
-        if (e != cudaSuccess) return fail(LSKUM_ERR_CUDA, std::string("dW: ") + cudaGetErrorString(e));
-        MLP_CUDA((k_colsum<<<blocks(N, 32), dim3(32, 8), 0, h->stream>>>(h->dZ, int(n), N, h->g + h->L.b_off[l]),
-                  cudaGetLastError()));
-        if (l == 0) break;
-        // dA_{l} [n x K] = dZ W_l : A(m = sample, k = out) = dZ, B(k = out, n = in) = W[out][in]
-        e = gemm<kStoreF32>(h, h->dZb, N, 1, h->L.W[l], K, 1, int(n), K, N, nullptr, h->dA, nullptr, K);
-        if (e != cudaSuccess) return fail(LSKUM_ERR_CUDA, std::string("dA: ") + cudaGetErrorString(e));
-        MLP_CUDA((k_tanh_back<<<blocks(n * K, 256), 256, 0, h->stream>>>(h->dA, h->Af[l], n * K, h->dZ, h->dZb),
-                  cudaGetLastError()));
+    const int64_t tiles = (n + kFwdRows - 1) / kFwdRows;
+    const unsigned grid = unsigned(std::min<int64_t>(tiles, h->sms));
+    BwdArgs b;
+    DwArgs w;
+    b.Y = h->Af[kLayers];
+    b.T = T;
+    for (int l = 0; l < kLayers; ++l) {
+        b.Af[l] = h->Af[l];
+        b.dZb[l] = h->dZb[l];
+        w.dZb[l] = h->dZb[l];
+        w.X[l] = h->Ab[l];
     }
+    b.Wt = h->Wt;
+    b.W5 = h->L.W[kLayers - 1];
+    b.sums = h->sums;
+    b.sq = h->partial;
+    w.L = h->L;
+    w.part = h->slices;
+    w.np = h->nparam;
+    k_backward<<<grid, kFwdThreads, kFwdSmem, h->stream>>>(b, n, h->err);
+    MLP_CUDA(cudaGetLastError());
+    const int kchunk = grad_kchunk(n), slices = int((n + kchunk - 1) / kchunk);
+    k_weight_grads<<<dim3(4, kLayers, slices), 256, kDwSmem, h->stream>>>(w, int(n), kchunk);
+    MLP_CUDA(cudaGetLastError());
+    k_reduce_grads<<<blocks(h->nparam, 256), 256, 0, h->stream>>>(w, slices, h->sums, h->partial, int(grid) * 4,
+                                                                  double(n * kOut), h->g, h->loss_dev);
+    MLP_CUDA(cudaGetLastError());
     return LSKUM_OK;
 }
 
@@ -969,6 +1057,7 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
     h->nparam = lskum_mlp_num_params();
     auto bail = [&](cudaError_t e) {
         for (void* p : h->allocs) cudaFree(p);
+        if (h->err) cudaFreeHost(h->err);
         if (h->own_stream) cudaStreamDestroy(h->own_stream);
         delete h;
         return fail(LSKUM_ERR_CUDA, std::string("lskum_mlp_create: ") + cudaGetErrorString(e));
@@ -976,6 +1065,10 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking)) != cudaSuccess) return bail(e);
     h->stream = h->own_stream;
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return bail(e);
     int64_t off = 0;
     for (int l = 0; l < kLayers; ++l) {
         h->L.w_off[l] = off;
@@ -986,20 +1079,31 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
     }
     if ((e = alloc(h, &h->p, h->nparam)) != cudaSuccess || (e = alloc(h, &h->g, h->nparam)) != cudaSuccess ||
         (e = alloc(h, &h->m, h->nparam)) != cudaSuccess || (e = alloc(h, &h->v, h->nparam)) != cudaSuccess ||
-        (e = alloc(h, &h->proj, 16)) != cudaSuccess || (e = alloc(h, &h->dA, capacity * kWidth)) != cudaSuccess ||
-        (e = alloc(h, &h->dZ, capacity * kWidth)) != cudaSuccess ||
-        (e = alloc(h, &h->dZb, capacity * kWidth)) != cudaSuccess ||
-        (e = alloc(h, &h->slices, int64_t(kMaxSlices) * kWidth * kWidth)) != cudaSuccess ||
-        (e = alloc(h, &h->partial, int64_t(blocks(capacity * kOut, 256)))) != cudaSuccess ||
+        (e = alloc(h, &h->proj, 16)) != cudaSuccess ||
+        (e = alloc(h, &h->slices, kMaxSlices * (h->nparam + 4 * kOut * kWidth))) != cudaSuccess ||
+        (e = alloc(h, &h->sums, 4 * int64_t(h->sms) * (kBwdSums + kOut))) != cudaSuccess ||
+        (e = alloc(h, &h->partial, 4 * int64_t(h->sms))) != cudaSuccess ||
+        (e = alloc(h, &h->Wt, packed_offset_t(0, 0, 0))) != cudaSuccess ||
         (e = alloc(h, &h->loss_dev, 1)) != cudaSuccess ||
-        (e = alloc(h, &h->err_dev, 1)) != cudaSuccess ||
-        (e = cudaMemset(h->err_dev, 0, sizeof(int))) != cudaSuccess)
+        (e = alloc(h, &h->Wp, packed_offset(kLayers - 1, 0, 0))) != cudaSuccess ||
+        (e = cudaMallocHost(&h->err, sizeof(int))) != cudaSuccess)
+        return bail(e);
+    *h->err = 0;
+    if ((e = cudaFuncSetAttribute(k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_forward<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem)) !=
+            cudaSuccess)
         return bail(e);
     for (int l = 0; l <= kLayers; ++l) {
         const int w = l == 0 ? kIn : (l == kLayers ? kOut : kWidth);
         if ((e = alloc(h, &h->Af[l], capacity * w)) != cudaSuccess ||
             (e = alloc(h, &h->Ab[l], capacity * w)) != cudaSuccess)
             return bail(e);
+        if (l < kLayers && (e = alloc(h, &h->dZb[l], capacity * layer_out(l))) != cudaSuccess) return bail(e);
     }
     if ((e = cudaMemcpy(h->proj, proj, 16 * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(h->p, 0, sizeof(float) * h->nparam)) != cudaSuccess ||
@@ -1014,6 +1118,7 @@ void lskum_mlp_destroy(lskum_mlp* h) {
     if (!h) return;
     cudaStreamSynchronize(h->stream);
     for (void* p : h->allocs) cudaFree(p);
+    cudaFreeHost(h->err);
     cudaStreamDestroy(h->own_stream);
     delete h;
 }
@@ -1024,7 +1129,8 @@ int lskum_mlp_set_params(lskum_mlp* h, const float* params, int64_t n) {
     MLP_CUDA(cudaMemsetAsync(h->m, 0, sizeof(float) * n, h->stream));
     MLP_CUDA(cudaMemsetAsync(h->v, 0, sizeof(float) * n, h->stream));
     h->step = 0;
-    MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L),
+    MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L,
+                                                                                                      h->Wp, h->Wt),
               cudaGetLastError()));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
     return LSKUM_OK;
@@ -1049,10 +1155,11 @@ int lskum_mlp_predict(lskum_mlp* h, const float* feat, int64_t n, float* out) {
     if (!h || !feat || !out) return fail(LSKUM_ERR_INVALID_ARG, "lskum_mlp_predict: null");
     int rc = check_n(h, n);
     if (rc) return rc;
-    MLP_CUDA(cudaMemcpyAsync(h->Af[0], feat, sizeof(float) * n * kIn, cudaMemcpyDeviceToDevice, h->stream));
-    rc = forward(h, n);
-    if (rc) return rc;
-    MLP_CUDA(cudaMemcpyAsync(out, h->Af[kLayers], sizeof(float) * n * kOut, cudaMemcpyDeviceToDevice, h->stream));
+    float* to = reinterpret_cast<uintptr_t>(out) & 15 ? h->Af[kLayers] : out;  // 16-byte stores
+    const float* f = nullptr;
+    if ((rc = stage_features(h, feat, n, to, &f)) || (rc = forward(h, f, n, to, false))) return rc;
+    if (to != out)
+        MLP_CUDA(cudaMemcpyAsync(out, to, sizeof(float) * n * kOut, cudaMemcpyDeviceToDevice, h->stream));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
     return check_gemm_status(h);
 }
@@ -1062,8 +1169,10 @@ int lskum_mlp_gradients(lskum_mlp* h, const float* feat, const float* target, in
     if (!h || !feat || !target) return fail(LSKUM_ERR_INVALID_ARG, "lskum_mlp_gradients: null");
     int rc = check_n(h, n);
     if (rc) return rc;
-    MLP_CUDA(cudaMemcpyAsync(h->Af[0], feat, sizeof(float) * n * kIn, cudaMemcpyDeviceToDevice, h->stream));
-    if ((rc = forward(h, n)) || (rc = backward(h, target, n))) return rc;
+    const float* f = nullptr;
+    if ((rc = stage_features(h, feat, n, nullptr, &f)) || (rc = forward(h, f, n, h->Af[kLayers], true)) ||
+        (rc = backward(h, target, n)))
+        return rc;
     if (grads) MLP_CUDA(cudaMemcpyAsync(grads, h->g, sizeof(float) * h->nparam, cudaMemcpyDeviceToHost, h->stream));
     if (loss) MLP_CUDA(cudaMemcpyAsync(loss, h->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
@@ -1075,8 +1184,10 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, i
     if (!h || !feat || !target || !(lr > 0.f)) return fail(LSKUM_ERR_INVALID_ARG, "lskum_mlp_train_step: argument");
     int rc = check_n(h, n);
     if (rc) return rc;
-    MLP_CUDA(cudaMemcpyAsync(h->Af[0], feat, sizeof(float) * n * kIn, cudaMemcpyDeviceToDevice, h->stream));
-    if ((rc = forward(h, n)) || (rc = backward(h, target, n))) return rc;
+    const float* f = nullptr;
+    if ((rc = stage_features(h, feat, n, nullptr, &f)) || (rc = forward(h, f, n, h->Af[kLayers], true)) ||
+        (rc = backward(h, target, n)))
+        return rc;
     h->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f / (1.f - powf(b1, float(h->step)));
@@ -1084,7 +1195,8 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, i
     MLP_CUDA((k_adam<<<blocks(h->nparam, 256), 256, 0, h->stream>>>(h->p, h->g, h->m, h->v, h->nparam, lr, b1, b2,
                                                                      1e-8f, c1, c2),
               cudaGetLastError()));
-    MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L),
+    MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L,
+                                                                                                      h->Wp, h->Wt),
               cudaGetLastError()));
     if (loss) {
         MLP_CUDA(cudaMemcpyAsync(loss, h->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -1103,8 +1215,7 @@ int lskum_mlp_sync(lskum_mlp* h) {
 int lskum_mlp_set_gemm(lskum_mlp* h, int path) {
     if (!h || (path != LSKUM_MLP_GEMM_MMA_SYNC && path != LSKUM_MLP_GEMM_TCGEN05))
         return fail(LSKUM_ERR_INVALID_ARG, "lskum_mlp_set_gemm: unknown path");
-    MLP_CUDA(cudaStreamSynchronize(h->stream));
-    h->gemm_path = path;
+    MLP_CUDA(cudaStreamSynchronize(h->stream));  // both paths are the fused tcgen05 pass
     return LSKUM_OK;
 }
 
