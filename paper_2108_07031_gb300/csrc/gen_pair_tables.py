@@ -11,6 +11,11 @@ the derivative of the same polynomial, so one row serves both.
 first has 11 significant bits (its products with the reduction's integer, up
 to 13 bits, are exact).
 
+3. ln x by table, x = 2^e m: for m's top seven bits j, F_j = 1/(1 + (j +
+1/2)/128) rounded to eight significant bits (so that m F_j - 1 is exact in a
+float) and -ln F_j as a pair of floats; ln2 in three floats whose first has 12
+significant bits.
+
 Run: python gen_pair_tables.py  (writes pair_tables.h next to this file)
 """
 
@@ -90,6 +95,18 @@ def main(path=None):
         for j in range(n_exp):
             h, l = split(mp.mpf(2) ** (mp.mpf(j) / n_exp))
             f.write(f"    {{{h!r}f, {l!r}f}},\n")
+        f.write("};\n\n")
+        ln2_hi = mp.floor(mp.log(2) * 2 ** 12) / 2 ** 12
+        ln2_mid, ln2_lo = split(mp.log(2) - ln2_hi)
+        f.write("// {F_j, -ln F_j hi, lo, 0}\n")
+        f.write(f"constexpr float kPairLn2Hi = {float(ln2_hi)!r}f;\nconstexpr float kPairLn2Mid = {ln2_mid!r}f;\n"
+                f"constexpr float kPairLn2Lo = {ln2_lo!r}f;\n")
+        f.write("alignas(16) __device__ const float kPairLog[128][4] = {\n")
+        for j in range(128):
+            F = 1 / (1 + (mp.mpf(j) + mp.mpf(1) / 2) / 128)
+            F = mp.nint(F * 2 ** 8) / 2 ** 8  # in (1/2, 1]: eight bits
+            h, l = split(-mp.log(F))
+            f.write(f"    {{{float(F)!r}f, {h!r}f, {l!r}f, 0.0f}},\n")
         f.write("};\n\n}  // namespace lskum\n")
     print(f"wrote {path}: {len(rows)} pieces, error {float(worst):.1e}, derivative {float(worst_d):.1e}")
 

@@ -142,6 +142,7 @@ cudaError_t timed(lskum_ctx* c, int cls, F&& launch) {
 // blocks of the stage-1 flux kernel: one partial sum of the residue each
 int n_blocks(const lskum_ctx* c) {
     if (c->pairs) return int(pair_flux_blocks(c->g, c->block));
+    if (c->mixed) return int(mx_flux_blocks(c->g, c->block));
     return int((c->g.n + c->block - 1) / c->block);
 }
 
@@ -394,7 +395,9 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
     DevState& st = c->st;
     const size_t N = size_t(L.n) * size_t(c->C);  // (point, condition) pairs
     // block partials when C == 1
-    const int nb = 1 + int(c->pairs ? pair_flux_blocks(g, kDefaultBlock) : (L.n + kDefaultBlock - 1) / kDefaultBlock);
+    const int nb = 1 + int(c->pairs   ? pair_flux_blocks(g, kDefaultBlock)
+                           : c->mixed ? mx_flux_blocks(g, kDefaultBlock)
+                                      : (L.n + kDefaultBlock - 1) / kDefaultBlock);
     if (c->mixed) {
         if ((e = dev_alloc(c, &st.qhl[0], N)) != cudaSuccess ||
             (e = dev_alloc(c, &st.qhl[1], N)) != cudaSuccess ||

@@ -180,6 +180,7 @@ cudaError_t launch_ls_inner_mx(const DevGeom& g, const DevGeom32& g32, const D8f
 cudaError_t launch_flux_mx(int mode, const DevGeom& g, const DevGeom32& g32, const Physics& ph,
                            const DevState& st, const QHL* q_in, const D8f* dq, QHL* q_out,
                            int block, cudaStream_t s);
+int64_t mx_flux_blocks(const DevGeom& g, int block);  // its blocks for the cloud
 cudaError_t launch_q_from_U_mx(const DevGeom& g, const Physics& ph, const V4* U, QHL* q,
                                cudaStream_t s);
 cudaError_t launch_dq_to_user_mx(const DevGeom& g, const D8f* src, V8* dst_user, cudaStream_t s);

@@ -14,6 +14,7 @@
 
 #include "flux_fp64.cuh"
 #include "flux_pair.cuh"
+#include "pair_convert.cuh"
 
 namespace lskum {
 
@@ -27,31 +28,6 @@ constexpr int kClasses = 4;
 // Microseconds a launch, one thread / four: 5,120 points 185 / 70, 46,080
 // 417 / 251, 321,056 pairs 1,518 / 1,462, 600,138 985 / 1,138.
 constexpr int64_t kSplitPairs = 1 << 18;
-
-// x as a pair: the leading 24 bits truncated, the other 29 rounded to a float.
-// Integer operations only (the conversions between FP64 and FP32 run at the
-// FP64 pipe's rate). |x| below 2^-74 gives zero, above 2^127 or not finite NaN.
-__device__ __forceinline__ Pf split_pair(const double x) {
-    const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x));
-    const uint32_t mag = hi & 0x7fffffffu;
-    const uint32_t hb = (hi & 0x80000000u) | ((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu);
-    Pf r;
-    r.h = bitsf(hb);
-    r.l = rmul(__uint2float_rn(lo & 0x1fffffffu), bitsf((hb & 0xff800000u) - (52u << 23)));
-    if (mag - 0x3b500000u >= 0x0ca00000u) {  // exponent outside [-74, 127)
-        const bool small = mag < 0x3b500000u;
-        r.h = small ? 0.f : __int_as_float(0x7fc00000);
-        r.l = 0.f;
-    }
-    return r;
-}
-
-// The double equal to a float, by integer operations; zero gives 2^-127 and a
-// subnormal less than 2^-125 (next to FP64 roundings of the values here).
-__device__ __forceinline__ double widen(const float x) {
-    const uint32_t u = fbits(x);
-    return __hiloint2double(int((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), int(u << 29));
-}
 
 __device__ __forceinline__ double join(const Pf a) { return widen(a.h) + widen(a.l); }
 

@@ -1,0 +1,37 @@
+// Conversions between FP64 and floats by integer operations: the hardware's run
+// at the FP64 pipe's rate, 1/64 of the FP32 and integer pipes'.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "pair_math.cuh"
+
+namespace lskum {
+
+// x as a pair: the leading 24 bits truncated, the other 29 rounded to a float.
+// Integer operations only (the conversions between FP64 and FP32 run at the
+// FP64 pipe's rate). |x| below 2^-74 gives zero, above 2^127 or not finite NaN.
+__device__ __forceinline__ Pf split_pair(const double x) {
+    const uint32_t hi = uint32_t(__double2hiint(x)), lo = uint32_t(__double2loint(x));
+    const uint32_t mag = hi & 0x7fffffffu;
+    const uint32_t hb = (hi & 0x80000000u) | ((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu);
+    Pf r;
+    r.h = bitsf(hb);
+    r.l = rmul(__uint2float_rn(lo & 0x1fffffffu), bitsf((hb & 0xff800000u) - (52u << 23)));
+    if (mag - 0x3b500000u >= 0x0ca00000u) {  // exponent outside [-74, 127)
+        const bool small = mag < 0x3b500000u;
+        r.h = small ? 0.f : __int_as_float(0x7fc00000);
+        r.l = 0.f;
+    }
+    return r;
+}
+
+// The double equal to a float, by integer operations; subnormals give zero.
+__device__ __forceinline__ double widen(const float x) {
+    const uint32_t u = fbits(x), mag = u & 0x7fffffffu;
+    const bool zero = mag < 0x00800000u;
+    return __hiloint2double(int((u & 0x80000000u) | (zero ? 0u : (mag >> 3) + 0x38000000u)),
+                            zero ? 0 : int(u << 29));
+}
+
+}  // namespace lskum

@@ -1,5 +1,5 @@
-"""The FP64 flux kernel's two layouts (four threads or one thread a point, by the
-number of (point, condition) pairs) give the same bits: a batch large enough
+"""The two layouts of the flux kernels and of the mixed sweeps (four threads or one
+thread a point, by the number of (point, condition) pairs) give the same bits: a batch large enough
 for one thread a point against its conditions solved alone. Neighbour counts
 1-4 modulo the four classes, a wall, a far field and entries of both the
 pair form and FP64 all occur in these clouds."""
@@ -19,7 +19,8 @@ from paper_2108_07031_gb300 import lskum as L  # noqa: E402
 
 
 @pytest.mark.parametrize("n_c, n_r, conditions, opts", [
-    (130, 41, 64, {}), (46, 23, 256, dict(order=1, inner_iters=0)), (131, 47, 64, dict(outer_mode=0))])
+    (130, 41, 64, {}), (46, 23, 256, dict(order=1, inner_iters=0)), (131, 47, 64, dict(outer_mode=0)),
+    (130, 41, 64, dict(precision=L.MIXED)), (131, 47, 64, dict(precision=L.MIXED, outer_mode=0, gamma=1.3))])
 def test_both_layouts_agree_bitwise(n_c, n_r, conditions, opts):
     cloud = Cl.naca0012_cloud(n_c, n_r, shuffle=True, seed=5)
     assert cloud.n <= 1 << 18 < cloud.n * conditions
