@@ -39,175 +39,8 @@ struct LayerPtrs {
     __nv_bfloat16* W[kLayers];
 };
 
-__device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};\n"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// Pipelined GEMM tile: 128 x 128 outputs a block of eight warps (each 64 x 32),
-// k in stages of 32 moved global -> shared by cp.async (16-byte chunks, three
-// stages in flight), operand fragments by ldmatrix -- plain for an operand whose
-// contraction index is contiguous in memory, transposed for one whose row index
-// is (dZ^T and X in the weight gradient) -- and mma.sync m16n8k16. The
-// contiguous dimension of each operand is a multiple of 8 elements with
-// 16-byte aligned rows.
-constexpr int kTB = 128;
-constexpr int kTK = 32;
-constexpr int kStages = 3;
-
-template <bool KFAST>
-struct TileGeo {  // shared-memory tile: [rows][ld] bf16, 16 bytes of row padding
-    static constexpr int ld = KFAST ? kTK + 8 : kTB + 8;
-    static constexpr int elems = KFAST ? kTB * ld : kTK * ld;
-};
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return uint32_t(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-    const int n = valid ? 16 : 0;  // 0: the 16 bytes are zero-filled, nothing is read
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(n));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t r[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t r[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-
-constexpr size_t tc_smem_bytes(bool ak, bool bk) {
-    return sizeof(__nv_bfloat16) * kStages *
-           size_t((ak ? TileGeo<true>::elems : TileGeo<false>::elems) +
-                  (bk ? TileGeo<true>::elems : TileGeo<false>::elems));
-}
-
-template <bool AK, bool BK>
-__device__ __forceinline__ void gemm_tc_block(const __nv_bfloat16* __restrict__ A, int64_t sam, int64_t sak,
-                                              const __nv_bfloat16* __restrict__ B, int64_t sbk, int64_t sbn,
-                                              int M, int N, int kbeg, int kend, int m0, int n0,
-                                              float* __restrict__ Cf, int64_t ldc) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(smem_raw);
-    __nv_bfloat16* sB = sA + kStages * TileGeo<AK>::elems;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = (warp >> 2) * 64, wn = (warp & 3) * 32;
-    const int ktiles = kend > kbeg ? (kend - kbeg + kTK - 1) / kTK : 0;
-
-    // one stage: 512 16-byte chunks of each operand tile, two per thread
-    auto load_stage = [&](int stage, int kt) {
-        const int k0 = kbeg + kt * kTK;
-        __nv_bfloat16* a = sA + stage * TileGeo<AK>::elems;
-        __nv_bfloat16* b = sB + stage * TileGeo<BK>::elems;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int c = tid + i * 256;
-            if (AK) {
-                const int r = c >> 2, kc = (c & 3) * 8, gm = m0 + r, gk = k0 + kc;
-                const bool ok = gm < M && gk < kend;
-                cp_async16(smem_u32(a + r * TileGeo<AK>::ld + kc), ok ? A + int64_t(gm) * sam + gk : A, ok);
-            } else {
-                const int r = c >> 4, mc = (c & 15) * 8, gk = k0 + r, gm = m0 + mc;
-                const bool ok = gk < kend && gm < M;
-                cp_async16(smem_u32(a + r * TileGeo<AK>::ld + mc), ok ? A + int64_t(gk) * sak + gm : A, ok);
-            }
-            if (BK) {
-                const int r = c >> 2, kc = (c & 3) * 8, gn = n0 + r, gk = k0 + kc;
-                const bool ok = gn < N && gk < kend;
-                cp_async16(smem_u32(b + r * TileGeo<BK>::ld + kc), ok ? B + int64_t(gn) * sbn + gk : B, ok);
-            } else {
-                const int r = c >> 4, nc = (c & 15) * 8, gk = k0 + r, gn = n0 + nc;
-                const bool ok = gk < kend && gn < N;
-                cp_async16(smem_u32(b + r * TileGeo<BK>::ld + nc), ok ? B + int64_t(gk) * sbk + gn : B, ok);
-            }
-        }
-    };
-
-    float acc[4][4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
-
-#pragma unroll
-    for (int st = 0; st < kStages - 1; ++st) {
-        if (st < ktiles) load_stage(st, st);
-        cp_async_commit();
-    }
-    for (int kt = 0; kt < ktiles; ++kt) {
-        cp_async_wait<kStages - 2>();  // stage kt has landed (this thread's copies)
-        __syncthreads();                // ... everyone's; stage kt-1 is no longer read
-        const int nxt = kt + kStages - 1;
-        if (nxt < ktiles) load_stage(nxt % kStages, nxt);
-        cp_async_commit();
-        const __nv_bfloat16* a = sA + (kt % kStages) * TileGeo<AK>::elems;
-        const __nv_bfloat16* b = sB + (kt % kStages) * TileGeo<BK>::elems;
-#pragma unroll
-        for (int ks = 0; ks < kTK; ks += 16) {
-            uint32_t af[4][4], bfr[4][2];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (AK) {  // [m][k]: matrices (m 0-7 | 8-15) x (k 0-7 | 8-15)
-                    const int row = wm + i * 16 + (lane & 15), col = ks + (lane >> 4) * 8;
-                    ldsm_x4(smem_u32(a + row * TileGeo<AK>::ld + col), af[i]);
-                } else {   // [k][m], transposed on load
-                    const int row = ks + (lane & 7) + (lane >> 4) * 8;
-                    const int col = wm + i * 16 + ((lane >> 3) & 1) * 8;
-                    ldsm_x4_t(smem_u32(a + row * TileGeo<AK>::ld + col), af[i]);
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 4; j += 2) {  // two n8 fragments per ldmatrix
-                uint32_t r[4];
-                if (BK) {  // [n][k]
-                    const int row = wn + j * 8 + (lane & 7) + (lane >> 4) * 8;
-                    const int col = ks + ((lane >> 3) & 1) * 8;
-                    ldsm_x4(smem_u32(b + row * TileGeo<BK>::ld + col), r);
-                } else {   // [k][n], transposed on load
-                    const int row = ks + (lane & 7) + ((lane >> 3) & 1) * 8;
-                    const int col = wn + j * 8 + (lane >> 4) * 8;
-                    ldsm_x4_t(smem_u32(b + row * TileGeo<BK>::ld + col), r);
-                }
-                bfr[j][0] = r[0];
-                bfr[j][1] = r[1];
-                bfr[j + 1][0] = r[2];
-                bfr[j + 1][1] = r[3];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16_16816(acc[i][j], af[i], bfr[j]);
-        }
-    }
-    cp_async_wait<0>();
-
-    const int grp = lane >> 2, tig = lane & 3;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int m = m0 + wm + i * 16 + grp + ((r & 2) ? 8 : 0);
-                const int n = n0 + wn + j * 8 + tig * 2 + (r & 1);
-                if (m >= M || n >= N) continue;
-                Cf[int64_t(m) * ldc + n] = acc[i][j][r];
-            }
 }
 
 // ------------------------------------------------- fused forward pass
@@ -264,6 +97,16 @@ __host__ __device__ inline int64_t packed_offset_t(int l, int n, int k) {
            (n % 64 / 8) * 128 + (k % 8) * 16 + (n % 8) * 2;
 }
 
+// What the passes leave for one another, by tiles of 128 samples, with a tile's
+// 128 rows next to one another so that a warp's 32 rows are one access: 16-byte
+// granules of eight BF16 units (A_l, dZ_l) or of four FP32 ones (A_l for tanh'),
+// [tile][granule][row]. A BF16 tile is at the same time the MMA operand of the
+// weight gradients, whose contraction runs over the rows (core matrices of
+// eight rows of a granule). Rows past n are written too (dZ = 0 there).
+__host__ __device__ inline int64_t granule(int64_t tile, int per_tile, int g, int row) {
+    return (tile * per_tile + g) * kFwdRows + row;
+}
+
 // SM100 shared-memory matrix descriptor: bits [0,14) start address >> 4,
 // [16,30) leading-dimension byte offset >> 4, [32,46) stride-dimension byte
 // offset >> 4, [46,48) descriptor version 1, [61,64) layout 0 (no swizzle).
@@ -304,13 +147,17 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {  // arrives when the 
                  : "memory");
 }
 
-// A bulk copy of `bytes` from global to shared memory that completes on `bar`.
-__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+// A bulk copy of `bytes` from global to shared memory that counts on `bar`; and
+// with the arrival that expects it.
+__device__ __forceinline__ void bulk_copy_only(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
         "l"(src), "r"(bytes), "r"(bar)
         : "memory");
+}
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    bulk_copy_only(dst, src, bytes, bar);
 }
 
 // `steps` MMAs of K 16 of a 128-row A chunk (sbo 4096) and a 256-row B chunk into
@@ -346,7 +193,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
 
 // feat: n x 32 FP32; Wp: the operand images (packed_offset); p: the FP32
 // parameters (biases; L's offsets), W5: the output layer's BF16 weights 4 x 256.
-// out: n x 4. TRAIN: also Af[l], Ab[l] (n x 256) of the hidden layers, and Ab[0].
+// out: n x 4. TRAIN: also Af[l], Ab[l] of the hidden layers, and Ab[0], in granules.
 // *err receives 1 if a wait ran out (the outputs are then incomplete).
 struct FwdStore {
     float* Af[kLayers];
@@ -456,10 +303,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                 unsigned char* dst = smem + (row >> 3) * 4096 + half * 256 + (row & 7) * 16;
                 *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
                 *reinterpret_cast<uint4*>(dst + 128) = make_uint4(v[4], v[5], v[6], v[7]);
-                if (TRAIN && live) {
-                    uint4* o = reinterpret_cast<uint4*>(st.Ab[0] + m * kIn + half * 16);
+                if (TRAIN) {
+                    uint4* o = reinterpret_cast<uint4*>(st.Ab[0]) + granule(tile, kIn / 8, half * 2, row);
                     o[0] = make_uint4(v[0], v[1], v[2], v[3]);
-                    o[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                    o[kFwdRows] = make_uint4(v[4], v[5], v[6], v[7]);
                 }
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -509,14 +356,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                             y.w = fmaf(x, w5.w, y.w);
                         }
                     }
-                    if (TRAIN && live) {
-                        float4* of = reinterpret_cast<float4*>(st.Af[l + 1] + m * kWidth + c0);
-                        uint4* ob = reinterpret_cast<uint4*>(st.Ab[l + 1] + m * kWidth + c0);
+                    if (TRAIN) {
+                        float4* of = reinterpret_cast<float4*>(st.Af[l + 1]) + granule(tile, 64, c0 / 4, row);
+                        uint4* ob = reinterpret_cast<uint4*>(st.Ab[l + 1]) + granule(tile, 32, c0 / 8, row);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) of[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                        for (int j = 0; j < 8; ++j)
+                            of[j * kFwdRows] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            ob[j] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                            ob[j * kFwdRows] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
                     }
                 }
             }
@@ -544,10 +392,21 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
+// Sums over the lanes of v[0..31]: lane j ends with element j's in v[0].
+__device__ __forceinline__ void sum_lanes(float v[32], const int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const float keep = lane & o ? v[j + o] : v[j], give = lane & o ? v[j] : v[j + o];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+}
+
 // ------------------------------------------------- fused backward pass
 // The error signals of a 128-row tile from the output to the first layer in one
 // CTA, as k_forward runs forwards (8,192 samples: loss and gradients 659 us with
-// a launch for each layer's product, sum and tanh', now 204): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
+// a launch for each layer's product, sum and tanh', 173 as one): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
 // dZ_(l-1) = (dZ_l W_l) (1 - A_l^2) for l = 4..1 with the products on the tensor
 // cores. Stores each layer's dZ in BF16 (the weight gradients' operand), the
 // column sums of the FP32 dZ (the bias gradients; one row of partial sums for
@@ -557,8 +416,8 @@ constexpr int kBwdSums = kFwdHidden * kWidth;  // columns of a partial row; then
 struct BwdArgs {
     const float* Y;  // n x 4 outputs and targets
     const float* T;
-    const float* Af[kLayers];      // A_l, l = 1..5
-    __nv_bfloat16* dZb[kLayers];   // dZ_l, l = 0..4 (n x 256), 5 (n x 4)
+    const float* Af[kLayers];      // A_l, l = 1..5, in granules
+    __nv_bfloat16* dZb[kLayers];   // dZ_l, l = 0..4 in granules, 5 n x 4
     const unsigned char* Wt;       // transposed operand images
     const __nv_bfloat16* W5;       // 4 x 256
     float* sums;                   // [4 gridDim][kBwdSums + 4]
@@ -671,8 +530,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 }
-                const float* act = a.Af[l + 1] + m * kWidth;
-                __nv_bfloat16* to = a.dZb[l] + m * kWidth;
+                const float4* act = reinterpret_cast<const float4*>(a.Af[l + 1]) + granule(tile, 64, 0, row);
+                uint4* to = reinterpret_cast<uint4*>(a.dZb[l]) + granule(tile, 32, 0, row);
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
                     const int c0 = kc * 64 + half * 32;
@@ -689,8 +548,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                     uint32_t b[16];
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
-                        const float4 x = live ? *reinterpret_cast<const float4*>(act + c0 + j)
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 x = act[(c0 + j) / 4 * kFwdRows];
                         v[j] *= 1.0f - x.x * x.x;
                         v[j + 1] *= 1.0f - x.y * x.y;
                         v[j + 2] *= 1.0f - x.z * x.z;
@@ -710,20 +568,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                         mbar_arrive(a_ready + 8 * kc);
                     }
-                    if (live) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            reinterpret_cast<uint4*>(to + c0)[j] =
-                                make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
-                    }
-                    // the 32 rows' sums of 32 columns: lane j ends with column j
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                        for (int j = 0; j < o; ++j) {
-                            const float keep = lane & o ? v[j + o] : v[j], give = lane & o ? v[j] : v[j + o];
-                            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-                        }
+                    for (int j = 0; j < 4; ++j)
+                        to[(c0 / 8 + j) * kFwdRows] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
+                    sum_lanes(v, lane);  // the warp's 32 rows: lane j ends with column j
                     db[l][kc] += v[0];
                 }
             }
@@ -760,10 +608,14 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
     if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-// All weight gradients of a slice of the samples, dW_l = dZ_l^T X_l, in one launch:
-// blockIdx.y 0..3 the layers 1..4 (four 128 x 128 tiles), 4 the first layer (two
-// 128 x 32 ones), 5 the output layer. Slice z goes to part + z * np, a whole
-// parameter vector.
+// All weight gradients of a slice of the tiles, dW_l = dZ_l^T A_l, in one launch:
+// blockIdx.x 0..7 the layers 1..4 in halves of 128 outputs, 8 and 9 the first
+// layer's halves, 10 the output layer. Slice z goes to part + z * np, a whole
+// parameter vector. A tile's operands are contiguous (granules): one bulk copy
+// each, two tiles in flight, eight MMAs (M 128, N 256 or 32, K 16 rows) with both
+// operands' contraction index the slower one; the accumulator goes out once a
+// slice. Bound by the copies, 96 KB a tile and half layer from L2 (mma.sync tiles
+// that re-read both operands took 36 us for 8,192 samples).
 struct DwArgs {
     const __nv_bfloat16* dZb[kLayers];
     const __nv_bfloat16* X[kLayers];
@@ -771,67 +623,173 @@ struct DwArgs {
     float* part;
     int64_t np;
 };
+constexpr int kDwThreads = 192;  // four epilogue warps, an MMA and a copy warp
+constexpr int kDwA = 16 * kFwdRows * 16, kDwB = 32 * kFwdRows * 16;  // bytes a tile
+constexpr int kDwOffBar = 2 * (kDwA + kDwB);
+constexpr int kDwSmem = kDwOffBar + 64;
+static_assert(kDwSmem <= 227 * 1024, "one CTA's shared memory");
 
-__global__ void __launch_bounds__(256) k_weight_grads(const DwArgs a, int n, int kchunk) {
-    const int l = blockIdx.y < 4 ? blockIdx.y + 1 : blockIdx.y == 4 ? 0 : kLayers - 1;
-    const int kbeg = blockIdx.z * kchunk, kend = min(n, kbeg + kchunk);
-    float* part = a.part + int64_t(blockIdx.z) * a.np + a.L.w_off[l];
-    if (l == kLayers - 1) {  // 4 x 256: a thread a column, a quarter of the slice a block
-        const int q = (kend - kbeg + 3) / 4, s0 = kbeg + int(blockIdx.x) * q, s1 = min(kend, s0 + q);
-        float acc[kOut] = {0.f, 0.f, 0.f, 0.f};
-        const __nv_bfloat16* x = a.X[l] + threadIdx.x;
+__global__ void __launch_bounds__(kDwThreads, 1) k_weight_grads(const DwArgs a, int n, int tiles_per_slice,
+                                                                int* __restrict__ err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tiles = (n + kFwdRows - 1) / kFwdRows;
+    const int t0 = int(blockIdx.z) * tiles_per_slice, t1 = min(tiles, t0 + tiles_per_slice);
+    if (blockIdx.x == 10) {  // 4 x 256: a warp takes a granule's 8 columns, lanes the rows
+        constexpr int l = kLayers - 1;
+        const uint4* X = reinterpret_cast<const uint4*>(a.X[l]);
         const uint2* dz = reinterpret_cast<const uint2*>(a.dZb[l]);
-#pragma unroll 4
-        for (int s = s0; s < s1; ++s) {
-            const float xv = __bfloat162float(x[int64_t(s) * kWidth]);
-            const uint2 d = dz[s];
-            acc[0] = fmaf(xv, __uint_as_float(d.x << 16), acc[0]);
-            acc[1] = fmaf(xv, __uint_as_float(d.x & 0xffff0000u), acc[1]);
-            acc[2] = fmaf(xv, __uint_as_float(d.y << 16), acc[2]);
-            acc[3] = fmaf(xv, __uint_as_float(d.y & 0xffff0000u), acc[3]);
+        for (int g = warp; g < kWidth / 8; g += kDwThreads / 32) {
+            float v[32] = {};  // [output][column]
+            for (int t = t0; t < t1; ++t)
+#pragma unroll
+                for (int r = lane; r < kFwdRows; r += 32) {
+                    const int64_t m = int64_t(t) * kFwdRows + r;
+                    if (m >= n) continue;
+                    const uint4 x = X[granule(t, kWidth / 8, g, r)];
+                    const uint2 d = dz[m];
+                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ds[2] = {d.x, d.y};
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const uint32_t xw = xs[j % 8 / 2], dw = ds[j / 16];
+                        v[j] = fmaf(__uint_as_float(j & 1 ? xw & 0xffff0000u : xw << 16),
+                                    __uint_as_float(j & 8 ? dw & 0xffff0000u : dw << 16), v[j]);
+                    }
+                }
+            sum_lanes(v, lane);
+            a.part[int64_t(blockIdx.z) * a.np + a.L.w_off[l] + (lane / 8) * kWidth + g * 8 + lane % 8] = v[0];
         }
-        // the quarters' rows go after the vectors of the slices
-        float* to = a.part + int64_t(gridDim.z) * a.np + (int64_t(blockIdx.z) * 4 + blockIdx.x) * (kOut * kWidth);
-        for (int o = 0; o < kOut; ++o) to[o * kWidth + threadIdx.x] = acc[o];
         return;
     }
-    if (l == 0 && blockIdx.x >= 2) return;
-    const int K = layer_in(l);
-    gemm_tc_block<false, false>(a.dZb[l], 1, kWidth, a.X[l], K, 1, kWidth, K, kbeg, kend,
-                                l == 0 ? int(blockIdx.x) * kTB : int(blockIdx.x >> 1) * kTB,
-                                l == 0 ? 0 : int(blockIdx.x & 1) * kTB, part, K);
+    const int l = blockIdx.x < 8 ? int(blockIdx.x) / 2 + 1 : 0, half = blockIdx.x & 1;
+    const int K = layer_in(l), bytesB = K / 8 * kFwdRows * 16;
+    const uint32_t sA = smem_u32(smem), sB = sA + 2 * kDwA;
+    const uint32_t bar = sA + kDwOffBar, full = bar, empty = bar + 16, done = bar + 32, tslot = bar + 40;
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(full + 8 * i));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(empty + 8 * i));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(done));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
+    if (warp == 4) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;\n" ::"r"(tslot));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    uint32_t tmem;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
+    bool ok = true;
+    if (warp == 5) {  // copies
+        if (lane == 0) {
+            int i = 0;
+            for (int t = t0; t < t1; ++t, ++i) {
+                const int s = i & 1;
+                if (i >= 2) ok = mbar_wait(empty + 8 * s, uint32_t(i / 2 - 1) & 1u);
+                if (!ok) break;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(full + 8 * s),
+                             "r"(kDwA + bytesB)
+                             : "memory");
+                bulk_copy_only(sA + uint32_t(s * kDwA),
+                               reinterpret_cast<const uint4*>(a.dZb[l]) + granule(t, kWidth / 8, half * 16, 0), kDwA,
+                               full + 8 * s);
+                bulk_copy_only(sB + uint32_t(s * kDwB), reinterpret_cast<const uint4*>(a.X[l]) + granule(t, K / 8, 0, 0),
+                               bytesB, full + 8 * s);
+            }
+            for (int j = max(0, i - 2); j < i; ++j) ok = mbar_wait(full + 8 * (j & 1), uint32_t(j / 2) & 1u) && ok;
+        }
+    } else if (warp == 4) {  // MMAs: both operands with the contraction (rows) as the slower index
+        if (lane == 0) {
+            const uint32_t idesc = umma_idesc_bf16_f32(kFwdRows, K) | (1u << 15) | (1u << 16);
+            int i = 0;
+            for (int t = t0; t < t1 && ok; ++t, ++i) {
+                const int s = i & 1;
+                ok = mbar_wait(full + 8 * s, uint32_t(i / 2) & 1u);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                for (int ks = 0; ks < kFwdRows / 16; ++ks)
+                    asm volatile(
+                        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+                        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                        "l"(umma_desc(sA + uint32_t(s * kDwA + ks * 256), 128, kFwdRows * 16)),
+                        "l"(umma_desc(sB + uint32_t(s * kDwB + ks * 256), 128, kFwdRows * 16)), "r"(idesc),
+                        "r"(i + ks));
+                mma_commit(empty + 8 * s);
+            }
+            if (ok) mma_commit(done);
+        }
+    } else {  // the slice's sums: a thread a row (output unit)
+        ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
+        if (ok) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            float* to = a.part + int64_t(blockIdx.z) * a.np + a.L.w_off[l] + int64_t(half * 128 + warp * 32 + lane) * K;
+            for (int c = 0; c < K; c += 32) {
+                float v[32];
+                tmem_ld32(tmem + (uint32_t(warp * 32) << 16) + uint32_t(c), v);
+#pragma unroll
+                for (int j = 0; j < 32; j += 4)
+                    *reinterpret_cast<float4*>(to + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+        }
+    }
+    if (!ok && lane == 0) *err = 1;
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    __syncwarp();
+    if (warp == 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
 }
 
 // The gradient vector from the slices (in slice order) and the partial column
-// sums, and the loss: mean squared error.
+// sums, and the loss: mean squared error. The first kBiasBlocks blocks take 32
+// columns of the sums each (eight threads a column, added in order), the next
+// one the loss, the others 256 weights each.
+constexpr int kBiasBlocks = (kBwdSums + kOut + 31) / 32;
+
 __global__ void __launch_bounds__(256) k_reduce_grads(const DwArgs a, int slices, const float* __restrict__ sums,
                                                       const double* __restrict__ sq, int rows, double count,
                                                       float* __restrict__ g, double* __restrict__ loss) {
-    const int64_t e = int64_t(blockIdx.x) * 256 + threadIdx.x;
-    if (e == 0) {
-        double s = 0.0;
-        for (int r = 0; r < rows; ++r) s += sq[r];
-        *loss = s / count;
-    }
-    if (e >= a.np) return;
-    int l = kLayers - 1;
-    while (e < a.L.w_off[l]) --l;
-    float s = 0.f;
-    if (e < a.L.b_off[l]) {
-        if (l < kLayers - 1) {
-#pragma unroll 4
-            for (int z = 0; z < slices; ++z) s += a.part[int64_t(z) * a.np + e];
-        } else {
-            const float* p = a.part + int64_t(slices) * a.np + (e - a.L.w_off[l]);
-#pragma unroll 4
-            for (int z = 0; z < 4 * slices; ++z) s += p[int64_t(z) * (kOut * kWidth)];
-        }
-    } else {
-        const float* p = sums + (l < kLayers - 1 ? l * kWidth : kBwdSums) + (e - a.L.b_off[l]);
+    const int tid = threadIdx.x;
+    if (blockIdx.x < kBiasBlocks) {
+        __shared__ float part[8][32];
+        const int c = int(blockIdx.x) * 32 + tid % 32;
+        float s = 0.f;
+        if (c < kBwdSums + kOut) {
 #pragma unroll 8
-        for (int r = 0; r < rows; ++r) s += p[int64_t(r) * (kBwdSums + kOut)];
+            for (int r = tid / 32; r < rows; r += 8) s += sums[int64_t(r) * (kBwdSums + kOut) + c];
+        }
+        part[tid / 32][tid % 32] = s;
+        __syncthreads();
+        if (tid < 32 && c < kBwdSums + kOut) {
+            float t = 0.f;
+            for (int k = 0; k < 8; ++k) t += part[k][tid];
+            g[a.L.b_off[c / kWidth] + c % kWidth] = t;  // kBwdSums is a multiple of kWidth
+        }
+    } else if (blockIdx.x == kBiasBlocks) {
+        __shared__ double part[256];
+        double s = 0.0;
+        for (int r = tid; r < rows; r += 256) s += sq[r];
+        part[tid] = s;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (tid < o) part[tid] += part[tid + o];
+            __syncthreads();
+        }
+        if (tid == 0) *loss = part[0] / count;
+    } else {
+        const int64_t e = int64_t(blockIdx.x - kBiasBlocks - 1) * 256 + tid;
+        if (e >= a.np) return;
+        int l = kLayers - 1;
+        while (e < a.L.w_off[l]) --l;
+        if (e >= a.L.b_off[l]) return;  // a bias
+        float s = 0.f;
+#pragma unroll 8
+        for (int z = 0; z < slices; ++z) s += a.part[int64_t(z) * a.np + e];
+        g[e] = s;
     }
-    g[e] = s;
 }
 
 // Features: per sample raw (x, y, wall distance, M, alpha_deg) ->
@@ -909,7 +867,8 @@ struct lskum_mlp {
     float* v = nullptr;
     float* proj = nullptr;  // 8 x 2 Fourier projection
     int64_t step = 0;
-    // activations: Af[l] (FP32) and Ab[l] (BF16) for l = 0..kLayers (l = 0: features)
+    // activations in granules: Af[l] (FP32, l = 1..5) and Ab[l] (BF16, l = 0..5;
+    // l = 0: features); Af[0] staged features, Af[kLayers] outputs
     float* Af[kLayers + 1] = {nullptr};
     __nv_bfloat16* Ab[kLayers + 1] = {nullptr};
     __nv_bfloat16* dZb[kLayers] = {nullptr};  // error signals (BF16)
@@ -950,7 +909,6 @@ cudaError_t alloc(lskum_mlp* h, T** p, int64_t count) {
 inline unsigned blocks(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
 constexpr int kMaxSlices = 16;
-constexpr int kDwSmem = int(tc_smem_bytes(false, false));
 
 // After a synchronising call: LSKUM_ERR_TIMEOUT (and the flag cleared) if a
 // forward pass gave up one of its waits.
@@ -990,12 +948,6 @@ int stage_features(lskum_mlp* h, const float* feat, int64_t n, const float* out,
     return LSKUM_OK;
 }
 
-// Slices of the weight gradients' contraction over n samples: at most
-// kMaxSlices of at least 256 samples, whole k stages each.
-int grad_kchunk(int64_t n) {
-    return int(std::max<int64_t>(256, ((n + kMaxSlices - 1) / kMaxSlices + kTK - 1) / kTK * kTK));
-}
-
 // backward from targets T (device n x 4): gradients into h->g, loss into loss_dev
 int backward(lskum_mlp* h, const float* T, int64_t n) {
     const int64_t tiles = (n + kFwdRows - 1) / kFwdRows;
@@ -1019,10 +971,12 @@ int backward(lskum_mlp* h, const float* T, int64_t n) {
     w.np = h->nparam;
     k_backward<<<grid, kFwdThreads, kFwdSmem, h->stream>>>(b, n, h->err);
     MLP_CUDA(cudaGetLastError());
-    const int kchunk = grad_kchunk(n), slices = int((n + kchunk - 1) / kchunk);
-    k_weight_grads<<<dim3(4, kLayers, slices), 256, kDwSmem, h->stream>>>(w, int(n), kchunk);
+    // at most kMaxSlices slices of whole tiles
+    const int per_slice = int((tiles + kMaxSlices - 1) / kMaxSlices);
+    const int slices = int((tiles + per_slice - 1) / per_slice);
+    k_weight_grads<<<dim3(11, 1, slices), kDwThreads, kDwSmem, h->stream>>>(w, int(n), per_slice, h->err);
     MLP_CUDA(cudaGetLastError());
-    k_reduce_grads<<<blocks(h->nparam, 256), 256, 0, h->stream>>>(w, slices, h->sums, h->partial, int(grid) * 4,
+    k_reduce_grads<<<kBiasBlocks + 1 + blocks(h->nparam, 256), 256, 0, h->stream>>>(w, slices, h->sums, h->partial, int(grid) * 4,
                                                                   double(n * kOut), h->g, h->loss_dev);
     MLP_CUDA(cudaGetLastError());
     return LSKUM_OK;
@@ -1080,7 +1034,7 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
     if ((e = alloc(h, &h->p, h->nparam)) != cudaSuccess || (e = alloc(h, &h->g, h->nparam)) != cudaSuccess ||
         (e = alloc(h, &h->m, h->nparam)) != cudaSuccess || (e = alloc(h, &h->v, h->nparam)) != cudaSuccess ||
         (e = alloc(h, &h->proj, 16)) != cudaSuccess ||
-        (e = alloc(h, &h->slices, kMaxSlices * (h->nparam + 4 * kOut * kWidth))) != cudaSuccess ||
+        (e = alloc(h, &h->slices, kMaxSlices * h->nparam)) != cudaSuccess ||
         (e = alloc(h, &h->sums, 4 * int64_t(h->sms) * (kBwdSums + kOut))) != cudaSuccess ||
         (e = alloc(h, &h->partial, 4 * int64_t(h->sms))) != cudaSuccess ||
         (e = alloc(h, &h->Wt, packed_offset_t(0, 0, 0))) != cudaSuccess ||
@@ -1098,12 +1052,13 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
         (e = cudaFuncSetAttribute(k_forward<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem)) !=
             cudaSuccess)
         return bail(e);
+    const int64_t rows = (capacity + kFwdRows - 1) / kFwdRows * kFwdRows;  // whole tiles
     for (int l = 0; l <= kLayers; ++l) {
         const int w = l == 0 ? kIn : (l == kLayers ? kOut : kWidth);
-        if ((e = alloc(h, &h->Af[l], capacity * w)) != cudaSuccess ||
-            (e = alloc(h, &h->Ab[l], capacity * w)) != cudaSuccess)
+        if ((e = alloc(h, &h->Af[l], rows * w)) != cudaSuccess ||
+            (l < kLayers && (e = alloc(h, &h->Ab[l], rows * w)) != cudaSuccess))
             return bail(e);
-        if (l < kLayers && (e = alloc(h, &h->dZb[l], capacity * layer_out(l))) != cudaSuccess) return bail(e);
+        if (l < kLayers && (e = alloc(h, &h->dZb[l], rows * layer_out(l))) != cudaSuccess) return bail(e);
     }
     if ((e = cudaMemcpy(h->proj, proj, 16 * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(h->p, 0, sizeof(float) * h->nparam)) != cudaSuccess ||
