@@ -637,26 +637,24 @@ int lskum_eval_residual(lskum_ctx* c, double* R) {
 int lskum_eval_q_derivatives(lskum_ctx* c, double* qx, double* qy) {
     if (!c || !qx || !qy) return fail(LSKUM_ERR_INVALID_ARG, "null argument");
     if (!c->have_state) return fail(LSKUM_ERR_STATE, "no state set");
+    const size_t N = size_t(c->g.n) * c->C;
     if (!c->staging8) {
-        LSKUM_CUDA(dev_alloc(c, &c->staging8, size_t(c->g.n) * c->C));
+        LSKUM_CUDA(dev_alloc(c, &c->staging8, N));
     }
+    V4* dx = reinterpret_cast<V4*>(c->staging8);
+    V4* dy = dx + N;
     int dbuf = 0;
     int64_t launches = 0;
     cudaError_t e = run_q_derivatives(c, 0, false, &dbuf, &launches);
     if (e != cudaSuccess) return cuda_fail(e, "q-derivatives");
     if (c->mixed) {
-        LSKUM_CUDA(launch_dq_to_user_mx(c->g, c->st.dq32[dbuf], c->staging8, c->stream));
+        LSKUM_CUDA(launch_dq_to_user_mx(c->g, c->st.dq32[dbuf], dx, dy, c->stream));
     } else {
-        LSKUM_CUDA(launch_gather_v8(c->g, c->st.dq[dbuf], c->staging8, c->stream));
+        LSKUM_CUDA(launch_gather_dq(c->g, c->st.dq[dbuf], dx, dy, c->stream));
     }
-    std::vector<V8> h(size_t(c->g.n) * c->C);
-    LSKUM_CUDA(cudaMemcpyAsync(h.data(), c->staging8, sizeof(V8) * h.size(), cudaMemcpyDeviceToHost, c->stream));
+    LSKUM_CUDA(cudaMemcpyAsync(qx, dx, sizeof(V4) * N, cudaMemcpyDeviceToHost, c->stream));
+    LSKUM_CUDA(cudaMemcpyAsync(qy, dy, sizeof(V4) * N, cudaMemcpyDeviceToHost, c->stream));
     LSKUM_CUDA(cudaStreamSynchronize(c->stream));
-    for (size_t i = 0; i < h.size(); ++i)
-        for (int m = 0; m < 4; ++m) {
-            qx[4 * i + m] = h[i].x[m];
-            qy[4 * i + m] = h[i].y[m];
-        }
     return LSKUM_OK;
 }
 

@@ -417,13 +417,24 @@ __global__ void k_q_from_U(const DevGeom g, const Physics ph, const V4* __restri
     q[t] = qq;
 }
 
-template <typename T>
-__global__ void k_gather(const DevGeom g, const T* __restrict__ src, T* __restrict__ dst) {
+__global__ void k_gather(const DevGeom g, const V4* __restrict__ src, V4* __restrict__ dst) {
     const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t d = t >> g.cshift;
     if (d >= g.n) return;
     const int64_t cc = int64_t(uint32_t(t) & g.cmask);
     dst[cc * g.n + g.dev_to_user[d]] = src[t];
+}
+
+// Derivatives in the caller's order, q_x and q_y apart (n x 4 each a condition).
+__global__ void k_gather_dq(const DevGeom g, const V8* __restrict__ src, V4* __restrict__ qx,
+                            V4* __restrict__ qy) {
+    const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t d = t >> g.cshift;
+    if (d >= g.n) return;
+    const int64_t at = int64_t(uint32_t(t) & g.cmask) * g.n + g.dev_to_user[d];
+    const V8 s = src[t];
+    qx[at] = V4{s.x[0], s.x[1], s.x[2], s.x[3]};
+    qy[at] = V4{s.y[0], s.y[1], s.y[2], s.y[3]};
 }
 
 // Residue per condition (C > 1), phase 1: block b reduces a contiguous range
@@ -617,12 +628,12 @@ cudaError_t launch_q_from_U(const DevGeom& g, const Physics& ph, const V4* U, V4
 }
 
 cudaError_t launch_gather_v4(const DevGeom& g, const V4* src, V4* dst, cudaStream_t s) {
-    k_gather<V4><<<grid_nc(g, 256), 256, 0, s>>>(g, src, dst);
+    k_gather<<<grid_nc(g, 256), 256, 0, s>>>(g, src, dst);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather_v8(const DevGeom& g, const V8* src, V8* dst, cudaStream_t s) {
-    k_gather<V8><<<grid_nc(g, 256), 256, 0, s>>>(g, src, dst);
+cudaError_t launch_gather_dq(const DevGeom& g, const V8* src, V4* qx, V4* qy, cudaStream_t s) {
+    k_gather_dq<<<grid_nc(g, 256), 256, 0, s>>>(g, src, qx, qy);
     return cudaGetLastError();
 }
 

@@ -168,7 +168,7 @@ cudaError_t launch_get_prim(const DevGeom& g, const Physics& ph, const V4* U, V4
                             cudaStream_t s);
 cudaError_t launch_q_from_U(const DevGeom& g, const Physics& ph, const V4* U, V4* q, cudaStream_t s);
 cudaError_t launch_gather_v4(const DevGeom& g, const V4* src_dev, V4* dst_user, cudaStream_t s);
-cudaError_t launch_gather_v8(const DevGeom& g, const V8* src_dev, V8* dst_user, cudaStream_t s);
+cudaError_t launch_gather_dq(const DevGeom& g, const V8* src_dev, V4* qx_user, V4* qy_user, cudaStream_t s);
 cudaError_t launch_forces(const DevGeom& g, const Physics& ph, const DevState& st,
                           cudaStream_t s);
 
@@ -183,6 +183,6 @@ cudaError_t launch_flux_mx(int mode, const DevGeom& g, const DevGeom32& g32, con
 int64_t mx_flux_blocks(const DevGeom& g, int block);  // its blocks for the cloud
 cudaError_t launch_q_from_U_mx(const DevGeom& g, const Physics& ph, const V4* U, QHL* q,
                                cudaStream_t s);
-cudaError_t launch_dq_to_user_mx(const DevGeom& g, const D8f* src, V8* dst_user, cudaStream_t s);
+cudaError_t launch_dq_to_user_mx(const DevGeom& g, const D8f* src, V4* qx_user, V4* qy_user, cudaStream_t s);
 
 }  // namespace lskum

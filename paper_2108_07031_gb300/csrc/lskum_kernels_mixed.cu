@@ -815,16 +815,15 @@ __global__ void k_q_from_U_mx(const DevGeom g, const Physics ph, const V4* __res
     q[t] = split_hl(qn);
 }
 
-__global__ void k_dq_to_v8(const DevGeom g, const D8f* __restrict__ src, V8* __restrict__ dst) {
+__global__ void k_gather_dq_mx(const DevGeom g, const D8f* __restrict__ src, V4* __restrict__ qx,
+                               V4* __restrict__ qy) {
     const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t d = t >> g.cshift;
     if (d >= g.n) return;
-    const int64_t cc = int64_t(uint32_t(t) & g.cmask);
+    const int64_t at = int64_t(uint32_t(t) & g.cmask) * g.n + g.dev_to_user[d];
     const D8f s = src[t];
-    V8 o;
-    o.x[0] = s.x.x; o.x[1] = s.x.y; o.x[2] = s.x.z; o.x[3] = s.x.w;
-    o.y[0] = s.y.x; o.y[1] = s.y.y; o.y[2] = s.y.z; o.y[3] = s.y.w;
-    dst[cc * g.n + g.dev_to_user[d]] = o;
+    qx[at] = V4{s.x.x, s.x.y, s.x.z, s.x.w};
+    qy[at] = V4{s.y.x, s.y.y, s.y.z, s.y.w};
 }
 
 inline unsigned grid_for(int64_t n, int block) { return unsigned((n + block - 1) / block); }
@@ -909,8 +908,8 @@ cudaError_t launch_q_from_U_mx(const DevGeom& g, const Physics& ph, const V4* U,
     return cudaGetLastError();
 }
 
-cudaError_t launch_dq_to_user_mx(const DevGeom& g, const D8f* src, V8* dst_user, cudaStream_t s) {
-    k_dq_to_v8<<<grid_nc(g, 256), 256, 0, s>>>(g, src, dst_user);
+cudaError_t launch_dq_to_user_mx(const DevGeom& g, const D8f* src, V4* qx_user, V4* qy_user, cudaStream_t s) {
+    k_gather_dq_mx<<<grid_nc(g, 256), 256, 0, s>>>(g, src, qx_user, qy_user);
     return cudaGetLastError();
 }
 
