@@ -406,7 +406,7 @@ __device__ __forceinline__ void sum_lanes(float v[32], const int lane) {
 // ------------------------------------------------- fused backward pass
 // The error signals of a 128-row tile from the output to the first layer in one
 // CTA, as k_forward runs forwards (8,192 samples: loss and gradients 659 us with
-// a launch for each layer's product, sum and tanh', 173 as one): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
+// a launch for each layer's product, sum and tanh', now 131): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
 // dZ_(l-1) = (dZ_l W_l) (1 - A_l^2) for l = 4..1 with the products on the tensor
 // cores. Stores each layer's dZ in BF16 (the weight gradients' operand), the
 // column sums of the FP32 dZ (the bias gradients; one row of partial sums for
@@ -610,12 +610,16 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
 
 // All weight gradients of a slice of the tiles, dW_l = dZ_l^T A_l, in one launch:
 // blockIdx.x 0..7 the layers 1..4 in halves of 128 outputs, 8 and 9 the first
-// layer's halves, 10 the output layer. Slice z goes to part + z * np, a whole
-// parameter vector. A tile's operands are contiguous (granules): one bulk copy
-// each, two tiles in flight, eight MMAs (M 128, N 256 or 32, K 16 rows) with both
-// operands' contraction index the slower one; the accumulator goes out once a
-// slice. Bound by the copies, 96 KB a tile and half layer from L2 (mma.sync tiles
-// that re-read both operands took 36 us for 8,192 samples).
+// layer's halves. Slice z goes to part + z * np, a whole parameter vector, each
+// half in granules of four columns by output unit, so that a
+// warp's store of 32 units is one access. A tile's operands are contiguous
+// (granules): one bulk copy each, two tiles in flight, eight MMAs (M 128, N 256
+// or 32, K 16 rows) with both operands' contraction index the slower one; the
+// accumulator goes out once a slice. Meanwhile the epilogue's four warps take
+// the output layer's gradient by FP32 FMAs, three or four of its 32 column
+// granules a block: as blocks of their own those were the last to end. Bound by
+// the copies, 96 KB a tile and half layer from L2, in one wave of at most 150
+// blocks (8,192 samples 14 us; mma.sync tiles that re-read both operands 36).
 struct DwArgs {
     const __nv_bfloat16* dZb[kLayers];
     const __nv_bfloat16* X[kLayers];
@@ -635,32 +639,6 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_weight_grads(const DwArgs a, 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tiles = (n + kFwdRows - 1) / kFwdRows;
     const int t0 = int(blockIdx.z) * tiles_per_slice, t1 = min(tiles, t0 + tiles_per_slice);
-    if (blockIdx.x == 10) {  // 4 x 256: a warp takes a granule's 8 columns, lanes the rows
-        constexpr int l = kLayers - 1;
-        const uint4* X = reinterpret_cast<const uint4*>(a.X[l]);
-        const uint2* dz = reinterpret_cast<const uint2*>(a.dZb[l]);
-        for (int g = warp; g < kWidth / 8; g += kDwThreads / 32) {
-            float v[32] = {};  // [output][column]
-            for (int t = t0; t < t1; ++t)
-#pragma unroll
-                for (int r = lane; r < kFwdRows; r += 32) {
-                    const int64_t m = int64_t(t) * kFwdRows + r;
-                    if (m >= n) continue;
-                    const uint4 x = X[granule(t, kWidth / 8, g, r)];
-                    const uint2 d = dz[m];
-                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ds[2] = {d.x, d.y};
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const uint32_t xw = xs[j % 8 / 2], dw = ds[j / 16];
-                        v[j] = fmaf(__uint_as_float(j & 1 ? xw & 0xffff0000u : xw << 16),
-                                    __uint_as_float(j & 8 ? dw & 0xffff0000u : dw << 16), v[j]);
-                    }
-                }
-            sum_lanes(v, lane);
-            a.part[int64_t(blockIdx.z) * a.np + a.L.w_off[l] + (lane / 8) * kWidth + g * 8 + lane % 8] = v[0];
-        }
-        return;
-    }
     const int l = blockIdx.x < 8 ? int(blockIdx.x) / 2 + 1 : 0, half = blockIdx.x & 1;
     const int K = layer_in(l), bytesB = K / 8 * kFwdRows * 16;
     const uint32_t sA = smem_u32(smem), sB = sA + 2 * kDwA;
@@ -722,17 +700,42 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_weight_grads(const DwArgs a, 
             }
             if (ok) mma_commit(done);
         }
-    } else {  // the slice's sums: a thread a row (output unit)
+    } else {
+        const int g = int(blockIdx.x) + 10 * warp;  // 4 x 8 of the output layer's: lanes take the rows
+        if (g < kWidth / 8) {
+            constexpr int o = kLayers - 1;
+            const uint4* X = reinterpret_cast<const uint4*>(a.X[o]);
+            const uint2* dz = reinterpret_cast<const uint2*>(a.dZb[o]);
+            float v[32] = {};  // [output][column]
+            for (int t = t0; t < t1; ++t)
+#pragma unroll
+                for (int r = lane; r < kFwdRows; r += 32) {
+                    const int64_t m = int64_t(t) * kFwdRows + r;
+                    const uint4 x = X[granule(t, kWidth / 8, g, r)];
+                    const uint2 d = m < n ? dz[m] : make_uint2(0u, 0u);
+                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ds[2] = {d.x, d.y};
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const uint32_t xw = xs[j % 8 / 2], dw = ds[j / 16];
+                        v[j] = fmaf(__uint_as_float(j & 1 ? xw & 0xffff0000u : xw << 16),
+                                    __uint_as_float(j & 8 ? dw & 0xffff0000u : dw << 16), v[j]);
+                    }
+                }
+            sum_lanes(v, lane);
+            a.part[int64_t(blockIdx.z) * a.np + a.L.w_off[o] + (lane / 8) * kWidth + g * 8 + lane % 8] = v[0];
+        }
+        // the slice's sums: a thread an output unit
         ok = __all_sync(0xffffffffu, mbar_wait(done, 0));
         if (ok) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            float* to = a.part + int64_t(blockIdx.z) * a.np + a.L.w_off[l] + int64_t(half * 128 + warp * 32 + lane) * K;
+            float4* to = reinterpret_cast<float4*>(a.part + int64_t(blockIdx.z) * a.np + a.L.w_off[l] +
+                                                   int64_t(half) * 128 * K) + warp * 32 + lane;
             for (int c = 0; c < K; c += 32) {
                 float v[32];
                 tmem_ld32(tmem + (uint32_t(warp * 32) << 16) + uint32_t(c), v);
 #pragma unroll
                 for (int j = 0; j < 32; j += 4)
-                    *reinterpret_cast<float4*>(to + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                    to[(c + j) / 4 * 128] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
             }
         }
     }
@@ -788,7 +791,8 @@ __global__ void __launch_bounds__(256) k_reduce_grads(const DwArgs a, int slices
         float s = 0.f;
 #pragma unroll 8
         for (int z = 0; z < slices; ++z) s += a.part[int64_t(z) * a.np + e];
-        g[e] = s;
+        const int i = int(e - a.L.w_off[l]), K = layer_in(l), half = i / (128 * K), q = i % (128 * K);
+        g[l == kLayers - 1 ? e : a.L.w_off[l] + (half * 128 + q / 4 % 128) * K + q / 512 * 4 + q % 4] = s;
     }
 }
 
@@ -908,7 +912,7 @@ cudaError_t alloc(lskum_mlp* h, T** p, int64_t count) {
 
 inline unsigned blocks(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
-constexpr int kMaxSlices = 16;
+constexpr int kMaxSlices = 15;  // of ten blocks: one wave
 
 // After a synchronising call: LSKUM_ERR_TIMEOUT (and the flag cleared) if a
 // forward pass gave up one of its waits.
@@ -974,7 +978,7 @@ int backward(lskum_mlp* h, const float* T, int64_t n) {
     // at most kMaxSlices slices of whole tiles
     const int per_slice = int((tiles + kMaxSlices - 1) / kMaxSlices);
     const int slices = int((tiles + per_slice - 1) / per_slice);
-    k_weight_grads<<<dim3(11, 1, slices), kDwThreads, kDwSmem, h->stream>>>(w, int(n), per_slice, h->err);
+    k_weight_grads<<<dim3(10, 1, slices), kDwThreads, kDwSmem, h->stream>>>(w, int(n), per_slice, h->err);
     MLP_CUDA(cudaGetLastError());
     k_reduce_grads<<<kBiasBlocks + 1 + blocks(h->nparam, 256), 256, 0, h->stream>>>(w, slices, h->sums, h->partial, int(grid) * 4,
                                                                   double(n * kOut), h->g, h->loss_dev);
