@@ -461,21 +461,30 @@ __global__ void __launch_bounds__(512) k_residue_cond_p1(const DevGeom g, const 
     }
 }
 
-// Phase 2 (one block): sum the block partials of each condition in block
-// order, append sqrt(sum)/N per condition to the history.
-__global__ void __launch_bounds__(256) k_residue_cond_p2(const DevGeom g, const DevState st,
-                                                         int nblocks) {
-    const int64_t C = int64_t(1) << g.cshift;
+// Phase 2 (one block): sum the block partials of each condition, append
+// sqrt(sum)/N per condition to the history. The block's threads share out the
+// partials of a condition (every kCondSumThreads / C-th each, then their sums in
+// order): a chain of loads a condition took 14 us longer for 64 of them.
+constexpr int kCondSumThreads = 1024;  // at least the conditions
+
+__global__ void __launch_bounds__(kCondSumThreads) k_residue_cond_p2(const DevGeom g, const DevState st,
+                                                                     int nblocks) {
+    __shared__ double part[kCondSumThreads];
+    const int C = 1 << g.cshift, groups = kCondSumThreads >> g.cshift;
     const unsigned long long it = *st.iter_counter;
-    const int64_t slot = int64_t(it % (unsigned long long)(st.res_cap / C));
-    for (int64_t c = threadIdx.x; c < C; c += blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += st.cpartials[int64_t(b) * C + c];
+    const int c = threadIdx.x & (C - 1);
+    double s = 0.0;
+#pragma unroll 8
+    for (int b = threadIdx.x >> g.cshift; b < nblocks; b += groups) s += st.cpartials[int64_t(b) * C + c];
+    part[threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.x < C) {
+        s = 0.0;
+        for (int k = 0; k < groups; ++k) s += part[(k << g.cshift) + c];
         const double r = sqrt(s) / double(g.n);
-        st.res_hist[slot * C + c] = r;
+        st.res_hist[int64_t(it % (unsigned long long)(st.res_cap / C)) * C + c] = r;
         if (!isfinite(r)) atomicOr(st.status, 1);
     }
-    __syncthreads();
     if (threadIdx.x == 0) *st.iter_counter = it + 1;
 }
 
@@ -600,7 +609,7 @@ cudaError_t launch_residue(const DevState& st, int nblocks, int64_t n, cudaStrea
 
 cudaError_t launch_residue_cond(const DevGeom& g, const DevState& st, cudaStream_t s) {
     k_residue_cond_p1<<<kCondReduceBlocks, dim3(32, 16), 0, s>>>(g, st);
-    k_residue_cond_p2<<<1, 256, 0, s>>>(g, st, kCondReduceBlocks);
+    k_residue_cond_p2<<<1, kCondSumThreads, 0, s>>>(g, st, kCondReduceBlocks);
     return cudaGetLastError();
 }
 
