@@ -24,7 +24,8 @@ CUDA_SOURCES = ["lskum_kernels.cu", "lskum_kernels_pair.cu", "lskum_kernels_mixe
                 "mlp_kernels.cu"]
 HOST_SOURCES = ["lskum_setup.cpp"]
 HEADERS = ["lskum_internal.h", "lskum_kernels.cuh", "math_tables.h", "device_math.cuh",
-           "flux_fp64.cuh", "pair_math.cuh", "pair_convert.cuh", "flux_pair.cuh", "pair_tables.h"]
+           "flux_fp64.cuh", "pair_math.cuh", "pair_convert.cuh", "flux_pair.cuh",
+           "pair_tables.h", "flux_fixed.cuh", "fixed_tables.h"]
 
 
 def _nvcc() -> str:

@@ -12,6 +12,7 @@
 // its lanes; the stage update, the next stage's q-variables and the residue
 // stay FP64.
 
+#include "flux_fixed.cuh"
 #include "flux_fp64.cuh"
 #include "flux_pair.cuh"
 #include "pair_convert.cuh"
@@ -23,10 +24,10 @@ namespace {
 constexpr int kClasses = 4;
 // Up to this many (point, condition) pairs four threads share a point. One
 // thread a point leaves SMs idle on a small cloud (5,120 points: 40 blocks),
-// and blocks of 128 points whose entries are FP64 ones are too large a unit of
-// work to balance; beyond it the four-fold set-up of a point costs more.
-// Microseconds a launch, one thread / four: 5,120 points 185 / 70, 46,080
-// 417 / 251, 321,056 pairs 1,518 / 1,462, 600,138 985 / 1,138.
+// and blocks of 128 points whose entries all have large steps are too large a
+// unit of work to balance; beyond it the four-fold set-up of a point costs more.
+// Microseconds a launch, one thread / four: 5,120 points 156 / 55, 46,080
+// 232 / 170, 150,598 429 / 403, 321,438 638 / 684, 600,138 960 / 1,091.
 constexpr int64_t kSplitPairs = 1 << 18;
 
 __device__ __forceinline__ double join(const Pf a) { return widen(a.h) + widen(a.l); }
@@ -34,15 +35,34 @@ __device__ __forceinline__ double join(const Pf a) { return widen(a.h) + widen(a
 __device__ __forceinline__ Pf dx_of(const float4& c) { return Pf{c.x, c.y}; }
 __device__ __forceinline__ Pf dy_of(const float4& c) { return Pf{c.z, c.w}; }
 
-// ws dGs + wn dGn of entry k of point d in FP64, in the point's frame: what
-// k_flux adds for that entry.
+// The two states' split fluxes by primitive variables in FP64, for states that
+// the fixed-point form does not take: |S| or ln(rho beta^2.5) out of its tables.
+__device__ __noinline__ void general_diff(const double* tj, const double* t0, const bool local,
+                                          const double2 nn, const uint32_t sc, const uint32_t nc,
+                                          const double gm1_inv, double* ds, double* dn) {
+    Prim wj = q_to_prim<true>(tj[0], tj[1], tj[2], tj[3], gm1_inv);
+    Prim w0 = q_to_prim<true>(t0[0], t0[1], t0[2], t0[3], gm1_inv);
+    if (local) {
+        const double nx = nn.x, ny = nn.y, tx = ny, ty = -nx;
+        const double sj = wj.u * tx + wj.v * ty, nj = wj.u * nx + wj.v * ny;
+        const double s0 = w0.u * tx + w0.v * ty, n0 = w0.u * nx + w0.v * ny;
+        wj.u = sj; wj.v = nj;
+        w0.u = s0; w0.v = n0;
+    }
+    const int64_t sm = sc == 2u ? kSignBit : 0, nm = nc == 2u ? kSignBit : 0;
+    split_flux_diff(wj, w0, wj.u, wj.v, w0.u, w0.v, split_ab(wj, wj.u, sm), split_ab(w0, w0.u, sm), ds);
+    split_flux_diff(wj, w0, wj.v, wj.u, w0.v, w0.u, split_ab(wj, wj.v, nm), split_ab(w0, w0.v, nm), dn);
+}
+
+// ws dGs + wn dGn of entry k of point d to FP64's accuracy, in the point's frame:
+// what k_flux adds for that entry. 64 FP64 instructions and some 1,700 on the
+// integer pipe (flux_fixed.cuh), where k_flux's formulas take 230 FP64 ones.
 __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
                                            const V4* __restrict__ q_in, const DQP* __restrict__ dq,
                                            const int64_t t, const int k, double c[4]) {
     const int64_t d = t >> g.cshift;
     const int64_t at = int64_t(k) * g.stride + d;
     const uint32_t e = g.nbr[at];
-    const uint32_t sc = (e >> kIndexBits) & 3u, nc = (e >> (kIndexBits + 2)) & 3u;
     const int64_t jt = sidx(g, e & kIndexMask, uint32_t(t) & g.cmask);
     const V4 qi = ld4(q_in + t), qj = ld4(q_in + jt);
     double tj[4] = {qj.a, qj.b, qj.c, qj.d};
@@ -65,38 +85,27 @@ __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& 
         }
     }
     if (!modified_states(second, hx, hy, vj, vi, tj, t0)) return;
-    Prim wj = q_to_prim<true>(tj[0], tj[1], tj[2], tj[3], ph.gm1_inv);
-    Prim w0 = q_to_prim<true>(t0[0], t0[1], t0[2], t0[3], ph.gm1_inv);
-    if (g.flag[d] != LSKUM_INTERIOR) {
-        const double2 nn = g.nrm[d];
-        const double nx = nn.x, ny = nn.y, tx = ny, ty = -nx;
-        const double sj = wj.u * tx + wj.v * ty, nj = wj.u * nx + wj.v * ny;
-        const double s0 = w0.u * tx + w0.v * ty, n0 = w0.u * nx + w0.v * ny;
-        wj.u = sj; wj.v = nj;
-        w0.u = s0; w0.v = n0;
+    const uint32_t sc = e >> kIndexBits & 3u, nc = e >> (kIndexBits + 2) & 3u;
+    const bool local = g.flag[d] != LSKUM_INTERIOR;
+    const double2 nn = local ? g.nrm[d] : make_double2(0.0, 1.0);
+    double ds[4], dn[4];
+    if (!fixed_diff(tj, t0, local, nn.x, nn.y, sc == 2u, nc == 2u, ds, dn)) {
+        const double gj[4] = {tj[0], tj[1], tj[2], tj[3]}, g0[4] = {t0[0], t0[1], t0[2], t0[3]};
+        double rs[4], rn[4];
+        general_diff(gj, g0, local, nn, sc, nc, ph.gm1_inv, rs, rn);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            ds[m] = sc ? rs[m] : 0.0;
+            dn[m] = nc ? rn[m] : 0.0;
+        }
     }
     const float4 wp = gp.weight[at];
-    double dg[4];
-    if (sc) {
-        const int64_t nmask = sc == 1u ? 0 : kSignBit;
-        split_flux_diff(wj, w0, wj.u, wj.v, w0.u, w0.v, split_ab(wj, wj.u, nmask),
-                        split_ab(w0, w0.u, nmask), dg);
-        const double w = join(Pf{wp.x, wp.y});
-        c[0] = w * dg[0];
-        c[1] = w * dg[1];
-        c[2] = w * dg[2];
-        c[3] = w * dg[3];
-    }
-    if (nc) {
-        const int64_t nmask = nc == 1u ? 0 : kSignBit;
-        split_flux_diff(wj, w0, wj.v, wj.u, w0.v, w0.u, split_ab(wj, wj.v, nmask),
-                        split_ab(w0, w0.v, nmask), dg);
-        const double w = join(Pf{wp.z, wp.w});
-        c[0] = fma(w, dg[0], c[0]);
-        c[1] = fma(w, dg[2], c[1]);
-        c[2] = fma(w, dg[1], c[2]);
-        c[3] = fma(w, dg[3], c[3]);
-    }
+    // an entry outside a stencil has weight 0 there
+    const double ws = join(Pf{wp.x, wp.y}), wn = join(Pf{wp.z, wp.w});
+    c[0] = fma(wn, dn[0], ws * ds[0]);
+    c[1] = fma(wn, dn[2], ws * ds[1]);
+    c[2] = fma(wn, dn[1], ws * ds[2]);
+    c[3] = fma(wn, dn[3], ws * ds[3]);
 }
 
 // The pair-form part of one point's entries first, first + stride, ...: adds to

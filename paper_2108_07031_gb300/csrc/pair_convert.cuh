@@ -2,12 +2,30 @@
 // at the FP64 pipe's rate, 1/64 of the FP32 and integer pipes'.
 #pragma once
 
-#include <cuda_runtime.h>
-
 #include "pair_math.cuh"
 
 namespace lskum {
 
+LSKUM_HD uint64_t dword(double x) {
+#ifdef __CUDA_ARCH__
+    return uint64_t(__double_as_longlong(x));
+#else
+    uint64_t u;
+    std::memcpy(&u, &x, 8);
+    return u;
+#endif
+}
+LSKUM_HD double dvalue(uint64_t u) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(int64_t(u));
+#else
+    double x;
+    std::memcpy(&x, &u, 8);
+    return x;
+#endif
+}
+
+#ifdef __CUDACC__
 // x as a pair: the leading 24 bits truncated, the other 29 rounded to a float.
 // Integer operations only (the conversions between FP64 and FP32 run at the
 // FP64 pipe's rate). |x| below 2^-74 gives zero, above 2^127 or not finite NaN.
@@ -25,13 +43,21 @@ __device__ __forceinline__ Pf split_pair(const double x) {
     }
     return r;
 }
+#endif
 
 // The double equal to a float, by integer operations; subnormals give zero.
-__device__ __forceinline__ double widen(const float x) {
+LSKUM_HD double widen(const float x) {
     const uint32_t u = fbits(x), mag = u & 0x7fffffffu;
     const bool zero = mag < 0x00800000u;
-    return __hiloint2double(int((u & 0x80000000u) | (zero ? 0u : (mag >> 3) + 0x38000000u)),
-                            zero ? 0 : int(u << 29));
+    return dvalue(uint64_t((u & 0x80000000u) | (zero ? 0u : (mag >> 3) + 0x38000000u)) << 32 |
+                  (zero ? 0u : u << 29));
+}
+
+// x truncated to a float, for 2^-100 < |x| < 2^100; smaller ones give zero.
+LSKUM_HD float narrow(const double x) {
+    const uint64_t u = dword(x);
+    const uint32_t hi = uint32_t(u >> 32), mag = uint32_t((u & 0x7fffffffffffffffULL) >> 29) - 0xc0000000u;
+    return (hi & 0x7fffffffu) < 0x39b00000u ? 0.f : bitsf((hi & 0x80000000u) | (mag & 0x7fffffffu));
 }
 
 }  // namespace lskum
