@@ -49,7 +49,7 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // stream from L2 through a ring of four 32 KB slots (64 of a layer's 256 k
 // each, laid out beforehand as the operand image, one bulk copy a slot), and
 // a layer's products accumulate in 256 columns of tensor memory, two layers'
-// accumulators side by side. Eight warps turn the accumulators into the next
+// accumulators side by side. Sixteen warps turn the accumulators into the next
 // layer's operand (bias, tanh, BF16), 64 columns at a time; the MMAs of those
 // 64 k start as soon as they are written, so they run under the tanh of the
 // next 64. One warp issues the MMAs, one the copies. The 4-wide output layer
@@ -70,7 +70,10 @@ constexpr int kFwdSlots = 4;                // weight ring
 constexpr int kFwdSlotBytes = 256 * 64 * 2; // 256 outputs x 64 k
 constexpr int kFwdIn0Bytes = 256 * 32 * 2;  // the first layer's one chunk
 constexpr int kFwdChunks = 1 + 4 * 4;       // chunks of a tile: layer 0, then 4 each of 4 layers
-constexpr int kFwdEpi = 256;                // epilogue threads
+constexpr int kFwdParts = 4;                // threads of a row, 16 of a chunk's 64 columns each
+constexpr int kFwdCols = 64 / kFwdParts;
+constexpr int kFwdEpi = kFwdRows * kFwdParts;  // epilogue threads
+constexpr int kFwdMmaWarp = kFwdEpi / 32, kFwdCopyWarp = kFwdMmaWarp + 1;
 constexpr int kFwdThreads = kFwdEpi + 64;   // and the MMA and the copy warp
 constexpr int kFwdABytes = kFwdRows * 256 * 2;
 constexpr int kFwdHidden = kLayers - 1;
@@ -79,7 +82,7 @@ constexpr int kFwdOffRing = kFwdABytes;
 constexpr int kFwdOffBias = kFwdOffRing + kFwdSlots * kFwdSlotBytes;
 constexpr int kFwdOffW5 = kFwdOffBias + kFwdHidden * 256 * 4;
 constexpr int kFwdOffPart = kFwdOffW5 + 256 * 16;
-constexpr int kFwdOffBar = kFwdOffPart + kFwdRows * 16;
+constexpr int kFwdOffBar = kFwdOffPart + (kFwdParts - 1) * kFwdRows * 16;
 constexpr int kFwdSmem = kFwdOffBar + 128;
 static_assert(kFwdSmem <= 227 * 1024, "one CTA's shared memory");
 
@@ -172,7 +175,7 @@ __device__ __forceinline__ void mma_chunk(uint32_t acc, uint32_t A, uint32_t B, 
             "r"(idesc), "r"(int(add) + ks));
 }
 
-// tcgen05.ld of 32 consecutive FP32 accumulator columns of this thread's
+// tcgen05.ld of 32 (16) consecutive FP32 accumulator columns of this thread's
 // tensor-memory lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
     uint32_t r[32];
@@ -189,6 +192,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float v[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+        "%11, %12, %13, %14, %15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+          "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // feat: n x 32 FP32; Wp: the operand images (packed_offset); p: the FP32
@@ -224,11 +241,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(a_ready + 8 * i), "r"(kFwdEpi));
         }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(acc_ready));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(part_ready), "r"(kFwdRows));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(part_ready), "r"((kFwdParts - 1) * kFwdRows));
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    if (warp == 8) {
+    if (warp == kFwdMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(tslot));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
@@ -244,7 +261,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
     bool ok = true;
 
-    if (warp == 9) {  // weight copies
+    if (warp == kFwdCopyWarp) {  // weight copies
         if (lane == 0) {
             int64_t g = 0;  // chunk counter
             for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
@@ -262,7 +279,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             for (int64_t i = max(int64_t(0), g - kFwdSlots); i < g; ++i)
                 ok = mbar_wait(full + 8 * int(i % kFwdSlots), uint32_t(i / kFwdSlots) & 1u) && ok;
         }
-    } else if (warp == 8) {  // MMAs
+    } else if (warp == kFwdMmaWarp) {  // MMAs
         if (lane == 0) {
             int64_t g = 0, t = 0;
             for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
@@ -284,30 +301,26 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             }
         }
     } else {  // epilogue
-        const int quarter = warp & 3, half = warp >> 2;
+        const int quarter = warp & 3, part = warp >> 2;
         const int row = quarter * 32 + lane;  // of the tile; this thread's tensor-memory lane
         int64_t t = 0;
         for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++t) {
             const int64_t m = tile * kFwdRows + row;
             const bool live = m < n;
-            {   // the features as BF16: half a row a thread
-                uint32_t v[8];
-                const float4* f = reinterpret_cast<const float4*>(feat + m * kIn + half * 16);
+            {   // the features as BF16, eight a thread
+                static_assert(kIn / kFwdParts == 8, "a 16-byte granule");
+                uint32_t v[4];
+                const float4* f = reinterpret_cast<const float4*>(feat + m * kIn + part * 8);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < 2; ++i) {
                     const float4 x = live ? f[i] : make_float4(0.f, 0.f, 0.f, 0.f);
                     const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
                     v[2 * i] = *reinterpret_cast<const uint32_t*>(&a);
                     v[2 * i + 1] = *reinterpret_cast<const uint32_t*>(&b);
                 }
-                unsigned char* dst = smem + (row >> 3) * 4096 + half * 256 + (row & 7) * 16;
-                *reinterpret_cast<uint4*>(dst) = make_uint4(v[0], v[1], v[2], v[3]);
-                *reinterpret_cast<uint4*>(dst + 128) = make_uint4(v[4], v[5], v[6], v[7]);
-                if (TRAIN) {
-                    uint4* o = reinterpret_cast<uint4*>(st.Ab[0]) + granule(tile, kIn / 8, half * 2, row);
-                    o[0] = make_uint4(v[0], v[1], v[2], v[3]);
-                    o[kFwdRows] = make_uint4(v[4], v[5], v[6], v[7]);
-                }
+                const uint4 b = make_uint4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<uint4*>(smem + (row >> 3) * 4096 + part * 128 + (row & 7) * 16) = b;
+                if (TRAIN) reinterpret_cast<uint4*>(st.Ab[0])[granule(tile, kIn / 8, part, row)] = b;
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                 mbar_arrive(a_ready);
@@ -319,12 +332,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const float* bias = s_bias + l * 256;
                 for (int kc = 0; kc < 4; ++kc) {  // 64 columns: the next layer's chunk of k
-                    const int c0 = kc * 64 + half * 32;
-                    float v[32];
-                    tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t((l & 1) * 256 + c0), v);
-                    uint32_t b[16];
+                    const int c0 = kc * 64 + part * kFwdCols;
+                    float v[kFwdCols];
+                    tmem_ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t((l & 1) * 256 + c0), v);
+                    uint32_t b[kFwdCols / 2];
 #pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
+                    for (int j = 0; j < kFwdCols; j += 4) {
                         const float4 bj = *reinterpret_cast<const float4*>(bias + c0 + j);
                         v[j] = tanhf(v[j] + bj.x);
                         v[j + 1] = tanhf(v[j + 1] + bj.y);
@@ -338,7 +351,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                     if (l < kFwdHidden - 1) {
                         unsigned char* dst = smem + (row >> 3) * 4096 + (c0 >> 3) * 128 + (row & 7) * 16;
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
+                        for (int j = 0; j < kFwdCols / 8; ++j)
                             *reinterpret_cast<uint4*>(dst + j * 128) =
                                 make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
                         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -346,7 +359,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                         mbar_arrive(a_ready + 8 * kc);
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
+                        for (int j = 0; j < kFwdCols; ++j) {
                             const uint32_t w = b[j / 2];
                             const float x = __uint_as_float(j & 1 ? w & 0xffff0000u : w << 16);
                             const float4 w5 = s_w5[c0 + j];
@@ -360,28 +373,31 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                         float4* of = reinterpret_cast<float4*>(st.Af[l + 1]) + granule(tile, 64, c0 / 4, row);
                         uint4* ob = reinterpret_cast<uint4*>(st.Ab[l + 1]) + granule(tile, 32, c0 / 8, row);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
+                        for (int j = 0; j < kFwdCols / 4; ++j)
                             of[j * kFwdRows] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
+                        for (int j = 0; j < kFwdCols / 8; ++j)
                             ob[j * kFwdRows] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
                     }
                 }
             }
             if (!ok) break;
-            // the two column halves of a row (a thread of the second half writes its
+            // a row's parts are added by its first thread (another one writes its
             // next part only after every thread has passed the next tile's layers)
-            if (half == 1) {
-                s_part[row] = y;
+            if (part > 0) {
+                s_part[(part - 1) * kFwdRows + row] = y;
                 mbar_arrive(part_ready);
                 continue;
             }
             ok = __all_sync(0xffffffffu, mbar_wait(part_ready, uint32_t(t) & 1u));
             if (ok && live) {
-                const float4 z = s_part[row];
                 const float* b5 = p + L.b_off[kLayers - 1];
-                reinterpret_cast<float4*>(out)[m] = make_float4(y.x + z.x + b5[0], y.y + z.y + b5[1],
-                                                                y.z + z.z + b5[2], y.w + z.w + b5[3]);
+#pragma unroll
+                for (int i = 0; i < kFwdParts - 1; ++i) {
+                    const float4 z = s_part[i * kFwdRows + row];
+                    y = make_float4(y.x + z.x, y.y + z.y, y.z + z.z, y.w + z.w);
+                }
+                reinterpret_cast<float4*>(out)[m] = make_float4(y.x + b5[0], y.y + b5[1], y.z + b5[2], y.w + b5[3]);
             }
         }
     }
@@ -389,7 +405,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     __syncwarp();
-    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+    if (warp == kFwdMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
 // Sums over the lanes of v[0..31]: lane j ends with element j's in v[0].
@@ -401,6 +417,18 @@ __device__ __forceinline__ void sum_lanes(float v[32], const int lane) {
             const float keep = lane & o ? v[j + o] : v[j], give = lane & o ? v[j] : v[j + o];
             v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
+}
+
+// Of v[0..15] likewise: lanes j and j + 16 end with element j's.
+__device__ __forceinline__ void sum_lanes16(float v[16], const int lane) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const float keep = lane & o ? v[j + o] : v[j], give = lane & o ? v[j] : v[j + o];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
 // ------------------------------------------------- fused backward pass
@@ -444,7 +472,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
-    if (warp == 8) {
+    if (warp == kFwdMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(tslot));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
     }
@@ -458,7 +486,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
     asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem) : "r"(tslot));
     bool ok = true;
 
-    if (warp == 9) {  // weight copies
+    if (warp == kFwdCopyWarp) {  // weight copies
         if (lane == 0) {
             int64_t g = 0;
             for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
@@ -473,7 +501,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
             for (int64_t i = max(int64_t(0), g - kFwdSlots); i < g; ++i)
                 ok = mbar_wait(full + 8 * int(i % kFwdSlots), uint32_t(i / kFwdSlots) & 1u) && ok;
         }
-    } else if (warp == 8) {  // MMAs
+    } else if (warp == kFwdMmaWarp) {  // MMAs
         if (lane == 0) {
             int64_t g = 0;
             for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
@@ -491,7 +519,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
             }
         }
     } else {  // epilogue
-        const int quarter = warp & 3, half = warp >> 2;
+        const int quarter = warp & 3, part = warp >> 2;
         const int row = quarter * 32 + lane;
         const float scale = float(n * kOut);
         float db[kFwdHidden][4] = {};  // this lane's columns: layer, chunk
@@ -512,7 +540,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                                           2.0f * d.w / scale);
             const __nv_bfloat162 b01 = __floats2bfloat162_rn(dy.x, dy.y), b23 = __floats2bfloat162_rn(dy.z, dy.w);
             const float2 r01 = __bfloat1622float2(b01), r23 = __bfloat1622float2(b23);
-            if (half == 0) {
+            if (part == 0) {
                 sq += double(d.x) * d.x + double(d.y) * d.y + double(d.z) * d.z + double(d.w) * d.w;
                 db5.x += dy.x;
                 db5.y += dy.y;
@@ -534,20 +562,20 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                 uint4* to = reinterpret_cast<uint4*>(a.dZb[l]) + granule(tile, 32, 0, row);
 #pragma unroll
                 for (int kc = 0; kc < 4; ++kc) {
-                    const int c0 = kc * 64 + half * 32;
-                    float v[32];
+                    const int c0 = kc * 64 + part * kFwdCols;
+                    float v[kFwdCols];
                     if (i == 0) {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
+                        for (int j = 0; j < kFwdCols; ++j) {
                             const float4 w = s_w5[c0 + j];
                             v[j] = fmaf(r23.y, w.w, fmaf(r23.x, w.z, fmaf(r01.y, w.y, r01.x * w.x)));
                         }
                     } else {
-                        tmem_ld32(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(((i - 1) & 1) * 256 + c0), v);
+                        tmem_ld16(tmem + (uint32_t(quarter * 32) << 16) + uint32_t(((i - 1) & 1) * 256 + c0), v);
                     }
-                    uint32_t b[16];
+                    uint32_t b[kFwdCols / 2];
 #pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
+                    for (int j = 0; j < kFwdCols; j += 4) {
                         const float4 x = act[(c0 + j) / 4 * kFwdRows];
                         v[j] *= 1.0f - x.x * x.x;
                         v[j + 1] *= 1.0f - x.y * x.y;
@@ -561,7 +589,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                     if (l > 0) {
                         unsigned char* dst = smem + (row >> 3) * 4096 + (c0 >> 3) * 128 + (row & 7) * 16;
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
+                        for (int j = 0; j < kFwdCols / 8; ++j)
                             *reinterpret_cast<uint4*>(dst + j * 128) =
                                 make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
                         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -569,9 +597,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
                         mbar_arrive(a_ready + 8 * kc);
                     }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
+                    for (int j = 0; j < kFwdCols / 8; ++j)
                         to[(c0 / 8 + j) * kFwdRows] = make_uint4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
-                    sum_lanes(v, lane);  // the warp's 32 rows: lane j ends with column j
+                    sum_lanes16(v, lane);  // the warp's 32 rows: lanes j, j + 16 end with column j
                     db[l][kc] += v[0];
                 }
             }
@@ -582,8 +610,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
 #pragma unroll
         for (int l = 0; l < kFwdHidden; ++l)
 #pragma unroll
-            for (int kc = 0; kc < 4; ++kc) out[l * kWidth + kc * 64 + half * 32 + lane] = db[l][kc];
-        if (half == 0) {
+            for (int kc = 0; kc < 4; ++kc)
+                if (lane < kFwdCols) out[l * kWidth + kc * 64 + part * kFwdCols + lane] = db[l][kc];
+        if (part == 0) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 sq += __shfl_xor_sync(0xffffffffu, sq, o);
@@ -605,7 +634,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     __syncwarp();
-    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+    if (warp == kFwdMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
 // All weight gradients of a slice of the tiles, dW_l = dZ_l^T A_l, in one launch:
