@@ -1,7 +1,8 @@
 // FP64 device kernels of the q-LSKUM hot path (sm_103a).
 //
-// Mapping: one thread per point, points in Hilbert-curve order (set-up), so a
-// warp's 32 points and their stencils are spatially close. Per-slot data
+// Mapping: one thread per point (the sweeps: four, a component each), points in
+// Hilbert-curve order (set-up), so a warp's points and their stencils are
+// spatially close. Per-slot data
 // (packed neighbour entry, half offsets, least-squares weights) is slot-major
 // [slot][point]: consecutive threads read consecutive words (coalesced). The
 // gathered per-point records are AoS: q (32 B) and (q_x, q_y) (64 B), so a
@@ -19,8 +20,8 @@
 //               step and the stage-1 partial sums of the residue.
 //   residue   : fixed-order reduction of the partial sums (deterministic).
 //
-// The arithmetic is FP64 throughout. On GB300 the FP64 pipe, not HBM,
-// bounds the flux kernel.
+// The arithmetic is FP64 throughout, and the FP64 pipe, not HBM, bounds the flux
+// kernel; for gamma = 1.4 lskum_kernels_pair.cu has the flux off that pipe.
 
 #include <cmath>
 
@@ -118,7 +119,8 @@ __global__ void __launch_bounds__(BLOCK) k_ls_inner(const DevGeom g, const V8* _
 
 // ------------------------------------------------------- flux residual + RK
 
-template <int MODE, int BLOCK, bool G14>
+// Every gamma but 1.4, which k_flux_pair takes.
+template <int MODE, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics ph,
                                                 const DevState st, const V4* __restrict__ q_in,
                                                 const V8* __restrict__ dq, V4* __restrict__ q_out) {
@@ -160,8 +162,8 @@ __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics p
                 if (!modified_states(second, second ? g.hdx[at] : 0.0, second ? g.hdy[at] : 0.0,
                                      second ? dq[jt] : di, di, tj, t0))
                     continue;
-                Prim wj = q_to_prim<G14>(tj[0], tj[1], tj[2], tj[3], ph.gm1_inv);
-                Prim w0 = q_to_prim<G14>(t0[0], t0[1], t0[2], t0[3], ph.gm1_inv);
+                Prim wj = q_to_prim<false>(tj[0], tj[1], tj[2], tj[3], ph.gm1_inv);
+                Prim w0 = q_to_prim<false>(t0[0], t0[1], t0[2], t0[3], ph.gm1_inv);
                 if (local) {  // velocities into (s, n)
                     const double sj = wj.u * tx + wj.v * ty, nj = wj.u * nx + wj.v * ny;
                     const double s0 = w0.u * tx + w0.v * ty, n0 = w0.u * nx + w0.v * ny;
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics p
                 R[2] = rs * ty + rn * ny;
             }
         }
-        r2 = stage_epilogue<MODE, G14>(g, ph, st, t, d, fl, fixed, R, q_out);
+        r2 = stage_epilogue<MODE, false>(g, ph, st, t, d, fl, fixed, R, q_out);
     }
     if (MODE == 1) {
         if (g.cshift == 0) {  // one condition: fused block partial sums
@@ -544,30 +546,23 @@ cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* din,
     return cudaGetLastError();
 }
 
-template <int BLOCK, bool G14>
+template <int BLOCK>
 static void flux_dispatch(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                           const V4* q_in, const V8* dq, V4* q_out, cudaStream_t s) {
     const unsigned grid = grid_nc(g, BLOCK);
     switch (mode) {
-        case 0: k_flux<0, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 1: k_flux<1, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 2: k_flux<2, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 3: k_flux<3, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        default: k_flux<4, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 0: k_flux<0, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 1: k_flux<1, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 2: k_flux<2, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 3: k_flux<3, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        default: k_flux<4, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
     }
 }
 
 cudaError_t launch_flux(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                         const V4* q_in, const V8* dq, V4* q_out, int block, cudaStream_t s) {
-    // gamma = 1.4: log-free density (see q_to_prim)
-    const bool g14 = fabs(ph.gm1_inv - 2.5) < 1e-12;
-    if (block == 256) {
-        if (g14) flux_dispatch<256, true>(mode, g, ph, st, q_in, dq, q_out, s);
-        else flux_dispatch<256, false>(mode, g, ph, st, q_in, dq, q_out, s);
-    } else {
-        if (g14) flux_dispatch<kDefaultBlock, true>(mode, g, ph, st, q_in, dq, q_out, s);
-        else flux_dispatch<kDefaultBlock, false>(mode, g, ph, st, q_in, dq, q_out, s);
-    }
+    if (block == 256) flux_dispatch<256>(mode, g, ph, st, q_in, dq, q_out, s);
+    else flux_dispatch<kDefaultBlock>(mode, g, ph, st, q_in, dq, q_out, s);
     return cudaGetLastError();
 }
 
