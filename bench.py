@@ -193,21 +193,23 @@ def _fp64_peak():
         return {"error": str(e)}
 
 
-# Per-unit figures of the FP64 flux/update kernel (k_flux), from one ncu
-# capture of a stage launch on the 600,138-point cloud (8,338,298 neighbour
-# entries): 1.0688e9 DFMA, 0.2379e9 DADD and 0.5728e9 DMUL thread
-# instructions (predicated on) = 2.948e9 FP64 flops = 353.6 flops per
-# neighbour entry (225.4 FP64 instructions), and 438.0 MB of DRAM traffic
-# = 729.8 bytes per point.
-# Units of one launch: neighbour entries (flops) and points (bytes); both
-# scale in proportion with the cloud size. With this instruction mix a
-# saturated FP64 pipe reaches (2 DFMA + DADD + DMUL) / (2 (DFMA + DADD +
-# DMUL)) = 0.784 of the FMA peak (every FP64 instruction takes one issue
-# slot of the pipe).
-FLUX_FP64_FLOPS_PER_NEIGHBOUR = 353.6
-FLUX_FP64_INSTR_PER_NEIGHBOUR = 225.4  # DFMA + DADD + DMUL
-FLUX_DRAM_BYTES_PER_POINT = 729.8
-FLUX_FRAC_CEILING = 0.784
+# Per-unit figures of the FP64 path's flux/update kernel (k_flux_pair: float
+# pairs and 64-bit fixed point in place of the FP64 pipe), from one ncu capture
+# of a stage launch on the 2,499,952-point cloud (34,760,611 neighbour entries):
+# 16.872e9 FFMA, 37.185e9 FADD and 10.276e9 FMUL thread instructions (predicated
+# on) = 81.21e9 FP32 flops = 2,336 per neighbour entry, 1,851 FP32 instructions
+# of 2,162 instructions in all (2.3484e9 warp instructions x 32), 0.290e9 FP64
+# instructions (8.3 per entry), and 1,853.5 MB of DRAM traffic = 741.4 bytes per
+# point. Units of one launch: neighbour entries (flops) and points (bytes); both
+# scale about in proportion with the cloud size (coarser clouds have more of
+# their entries in fixed point). With this instruction mix a saturated FP32 pipe
+# reaches (2 FFMA + FADD + FMUL) / (2 (FFMA + FADD + FMUL)) = 0.631 of the FMA
+# peak.
+FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR = 2336.0
+FLUX_PAIR_INSTR_PER_NEIGHBOUR = 2162.0  # thread instructions, all pipes
+FLUX_DRAM_BYTES_PER_POINT = 741.4
+FLUX_FRAC_CEILING = 0.631
+ISSUE_PEAK = 152 * 4 * 32 * 2.07e9  # thread instructions per second, one a scheduler and clock
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12  # 1.2586
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12  # 80.55: 128 FP32 lanes per SM
 ALGORITHMIC_BYTES_PER_POINT_ITERATION = 4600.0  # minimal passes, gathers from cache
@@ -218,14 +220,14 @@ ALGORITHMIC_BYTES_PER_POINT_ITERATION = 4600.0  # minimal passes, gathers from c
 #   mixed: k_flux_mx, FP32 flops (2 FFMA + FADD + FMUL) per entry; its FP64
 #          epilogue (state update, q-variables) is per point;
 #   split: the four k_flux_part launches and k_stage_split of one stage.
-#   mixed: 0.7822e9 FFMA + 1.0223e9 FMUL + 0.5091e9 FADD = 3.096e9 FP32 flops
-#          = 371.3 per entry (plus 57 FP64 instructions per point), 277.0 MB
-#          of DRAM traffic = 461.6 bytes per point;
+#   mixed: 0.9051e9 FFMA + 0.9243e9 FMUL + 0.4576e9 FADD = 3.192e9 FP32 flops
+#          = 382.8 per entry (plus 13 FP64 instructions per point), 279.7 MB
+#          of DRAM traffic = 466.1 bytes per point;
 #   split: 1.4516e9 DFMA + 0.2950e9 DADD + 0.8724e9 DMUL over the five
 #          launches of a stage = 4.071e9 FP64 flops = 488.2 per entry,
 #          1353.9 MB = 2256 bytes per point.
-FLUX_MX_FP32_FLOPS_PER_NEIGHBOUR = 371.3
-FLUX_MX_DRAM_BYTES_PER_POINT = 461.6
+FLUX_MX_FP32_FLOPS_PER_NEIGHBOUR = 382.8
+FLUX_MX_DRAM_BYTES_PER_POINT = 466.1
 FLUX_SPLIT_FP64_FLOPS_PER_NEIGHBOUR = 488.2
 FLUX_SPLIT_DRAM_BYTES_PER_POINT = 2257.0
 
@@ -344,10 +346,10 @@ def run_ours(args, rank, world, local):
         peaks = _fp64_peak()
         nnz = int(cloud.nbr_offsets[-1])
         flux_launch_ms = flux_ms / max(flux_n, 1)
-        achieved = FLUX_FP64_FLOPS_PER_NEIGHBOUR * nnz / (flux_launch_ms * 1e-3) / 1e12
+        achieved = FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR * nnz / (flux_launch_ms * 1e-3) / 1e12
         # ALU-bound kernel: the peak derived from unit counts and clocks,
-        # 152 SMs x 2 FP64 FMA per SM per clock x 2 flops x 2.07 GHz
-        peak = FP64_PEAK_TFLOPS
+        # 152 SMs x 128 FP32 FMA per SM per clock x 2 flops x 2.07 GHz
+        peak = FP32_PEAK_TFLOPS
         mp, mp_kind = _peaks()
         cpu = cpu_baseline(args) if not args.no_cpu_baseline else None
         result = {
@@ -358,22 +360,23 @@ def run_ours(args, rank, world, local):
             "config": config,
             "max_neighbours": info["max_neighbours"],
             "roofline": {
-                "kernel": "k_flux (flux residual + SSP-RK stage update, FP64)", "bound": "alu",
+                "kernel": "k_flux_pair (flux residual + SSP-RK stage update, FP64 path in float pairs)",
+                "bound": "alu",
                 "unit": "TFLOP/s", "achieved": achieved, "peak": peak,
                 "frac": (achieved / peak) if peak else None,
                 "traffic": FLUX_DRAM_BYTES_PER_POINT * n,
-                "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk/SM x 2 flops x 2.07 GHz "
+                "peak_source": "derived: 152 SMs x 128 FP32 FMA/clk/SM x 2 flops x 2.07 GHz "
                                "(maximum SM clock)",
-                "measured_fma_peak": peaks.get("fp64_fma_tflops"),
-                "measured_fma_peak_source": "pure-DFMA probe (pipe_peaks) run live on this GPU",
-                "flops_per_launch": FLUX_FP64_FLOPS_PER_NEIGHBOUR * nnz,
+                "measured_fp64_fma_peak": peaks.get("fp64_fma_tflops"),
+                "measured_fp64_fma_peak_source": "pure-DFMA probe (pipe_peaks) run live on this GPU",
+                "flops_per_launch": FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR * nnz,
                 "frac_ceiling_at_instruction_mix": FLUX_FRAC_CEILING,
-                # the pipe's own bound: FP64 instructions issued per second
-                # against 152 SMs x 2 per clock x 2.07 GHz
-                "fp64_issue_frac": (FLUX_FP64_INSTR_PER_NEIGHBOUR * nnz / (flux_launch_ms * 1e-3))
-                                   / (FP64_PEAK_TFLOPS * 1e12 / 2) if flux_launch_ms else None,
+                # the schedulers' own bound: instructions issued per second
+                # against one per scheduler and clock
+                "issue_frac": (FLUX_PAIR_INSTR_PER_NEIGHBOUR * nnz / (flux_launch_ms * 1e-3))
+                              / ISSUE_PEAK if flux_launch_ms else None,
                 "launch_ms": flux_launch_ms,
-                "traffic_note": "ncu dram bytes of a 0.6M-point launch scaled by points",
+                "traffic_note": "ncu dram bytes of a 2.5M-point launch scaled by points",
                 "hbm_frac_of_measured_whole_step": {
                     "algorithmic": (ALGORITHMIC_BYTES_PER_POINT_ITERATION * n
                                     / (t_max / args.steps * 1e-3)) / (mp["hbm_gbs"] * 1e9),
@@ -500,8 +503,8 @@ def time_variant(args, cloud, precision, n_cond, stream, barrier, dist, what,
 
 def variant_roofline(mixed: bool, split: bool, flux_time, nnz: int, n: int, n_cond: int,
                      ms_per_step: float) -> dict:
-    """Roofline of a variant's dominant kernel (the flux kernel: FP32 issue
-    for the mixed path, the FP64 pipe otherwise) and the HBM fraction of its
+    """Roofline of a variant's dominant kernel (the flux kernel: FP32 pipes,
+    the FP64 pipe for the split ablation) and the HBM fraction of its
     whole step, both from the live CUDA-event times of the timed region."""
     flux_ms, flux_n = flux_time
     launch_s = flux_ms / max(flux_n, 1) * 1e-3
@@ -515,9 +518,10 @@ def variant_roofline(mixed: bool, split: bool, flux_time, nnz: int, n: int, n_co
                                         FLUX_SPLIT_DRAM_BYTES_PER_POINT)
         peak, peak_src = FP64_PEAK_TFLOPS, "derived: 152 SMs x 2 FP64 FMA/clk/SM x 2 flops x 2.07 GHz"
     else:
-        kernel, per_entry, per_point = ("k_flux (flux residual + SSP-RK stage update, FP64)",
-                                        FLUX_FP64_FLOPS_PER_NEIGHBOUR, FLUX_DRAM_BYTES_PER_POINT)
-        peak, peak_src = FP64_PEAK_TFLOPS, "derived: 152 SMs x 2 FP64 FMA/clk/SM x 2 flops x 2.07 GHz"
+        # of small steps throughout; a coarse cloud's entries in fixed point count as theirs
+        kernel, per_entry, per_point = ("k_flux_pair (flux residual + stage update, FP64 path in float pairs)",
+                                        FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR, FLUX_DRAM_BYTES_PER_POINT)
+        peak, peak_src = FP32_PEAK_TFLOPS, "derived: 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz"
     achieved = per_entry * nnz * n_cond / launch_s / 1e12 if per_entry else None
     mp, mp_kind = _peaks()
     hbm = mp["hbm_gbs"] * 1e9
