@@ -58,10 +58,12 @@ extern "C" {
 #define LSKUM_MAX_NEIGHBOURS 20
 
 /* Precision modes. */
-#define LSKUM_FP64 0  /* every step in FP64 */
+#define LSKUM_FP64 0  /* every step in FP64, or to its accuracy in float pairs and
+                         64-bit fixed point (the fluxes of gamma = 1.4) */
 #define LSKUM_MIXED 1 /* FP32 stencil, least-squares and split-flux arithmetic (in
-                         difference form, on q stored as float pairs); FP64 state
-                         accumulation, q-variables, LS determinants, residue, forces */
+                         difference form, on q stored as float pairs); q-variables
+                         in float pairs; FP64 state accumulation, LS determinants,
+                         residue, forces */
 
 /* Outer-boundary modes. */
 #define LSKUM_OUTER_FREESTREAM 1 /* far-field points hold the free-stream state */

@@ -14,7 +14,7 @@ CSRC = os.path.join(ROOT, "paper_2108_07031_gb300", "csrc")
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def measured(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("flux_fixed") / "check")
     subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-o", exe,
                     os.path.join(ROOT, "tests", "flux_pair", "check_flux_fixed.cpp")]
@@ -29,19 +29,19 @@ def checker(tmp_path_factory):
 
 @pytest.mark.parametrize("mach", [0.0, 0.3, 0.85, 2.0, 4.5])
 @pytest.mark.parametrize("log2_step", [-30, -6, -3, 0])
-def test_difference_error(checker, mach, log2_step):
+def test_difference_error(measured, mach, log2_step):
     """Factors, moments, the first product and the difference are each rounded
     once, by half of 2^-52 at most: 2^-52 of G in the 2-norm. A plain double
     evaluation with a moving gas is no nearer."""
-    taken, err, err64 = checker(mach, log2_step)
+    taken, err, err64 = measured(mach, log2_step)
     assert taken == 2000 or (mach == 4.5 and taken > 1500)
     assert max(err) < 2.0 ** -52
     assert mach == 0.0 or all(a <= b for a, b in zip(err, err64))
 
 
-def test_states_out_of_range_are_left_out(checker):
+def test_states_out_of_range_are_left_out(measured):
     """|S| beyond the table of erfcx (most states at Mach 40): refused."""
-    assert checker(40.0, 0)[0] < 60
+    assert measured(40.0, 0)[0] < 60
 
 
 def test_tables_match_their_generator(tmp_path):

@@ -14,7 +14,7 @@ CSRC = os.path.join(ROOT, "paper_2108_07031_gb300", "csrc")
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def measured(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("flux_pair") / "check")
     subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-o", exe,
                     os.path.join(ROOT, "tests", "flux_pair", "check_flux_pair.cpp")]
@@ -29,12 +29,12 @@ def checker(tmp_path_factory):
 
 @pytest.mark.parametrize("mach", [0.0, 0.3, 0.85, 2.0])
 @pytest.mark.parametrize("log2_step", [-20, -12, -8, -7])
-def test_difference_error(checker, mach, log2_step):
+def test_difference_error(measured, mach, log2_step):
     """About a hundred pair operations of 2^-47 each stand behind a component:
     2^-43 of dG in the 2-norm; and no further off than the double evaluation,
     which is left with 2^-51.5 / step (in still air state 0 has no momentum to
     cancel, so double has nothing to lose there)."""
-    taken, err, err64 = checker(mach, log2_step)
+    taken, err, err64 = measured(mach, log2_step)
     # beyond Mach 1 ln(rho beta^2.5) moves by many times the step
     assert taken == 2000 or (log2_step == -7 and taken > 1000)
     assert max(err) < 2.0 ** -43
@@ -42,10 +42,10 @@ def test_difference_error(checker, mach, log2_step):
 
 
 @pytest.mark.parametrize("mach, log2_step", [(0.63, -1), (40.0, -20)])
-def test_large_steps_and_states_out_of_range_are_left_out(checker, mach, log2_step):
+def test_large_steps_and_states_out_of_range_are_left_out(measured, mach, log2_step):
     """Steps over the limits, and |S| beyond the table of Phi (most pairs at
     Mach 40): the form refuses them."""
-    assert checker(mach, log2_step)[0] < 60
+    assert measured(mach, log2_step)[0] < 60
 
 
 def test_tables_match_their_generator(tmp_path):
