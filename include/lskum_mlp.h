@@ -11,9 +11,8 @@
  * Network: 21 input features (zero-padded to LSKUM_MLP_IN_PADDED) -> five
  * hidden layers of LSKUM_MLP_WIDTH (tanh) -> LSKUM_MLP_OUT linear outputs
  * (six linear layers). Training and inference run in hand-written CUDA
- * kernels: BF16 tensor-core products (tcgen05 for the fused forward and
- * backward passes, mma.sync m16n8k16 for the weight gradients) accumulating
- * in FP32, FP32 master weights, Adam.
+ * kernels: BF16 tensor-core products (tcgen05: the fused forward and backward
+ * passes, the weight gradients) accumulating in FP32, FP32 master weights, Adam.
  *
  * Parameters (flat FP32, host order): for l = 0..5: W_l [out_l x in_l]
  * row-major, then b_l [out_l]; in_0 = LSKUM_MLP_IN_PADDED (columns 21..31
@@ -86,9 +85,8 @@ int lskum_mlp_sync(lskum_mlp* h);
 
 /* GEMM path of the forward pass's five 256-wide layers. Both values select the
  * fused pass on the fifth-generation tensor cores (tcgen05.mma M 128, N 256,
- * K 16 into tensor memory, all layers of 128 samples in one CTA), which gives
- * the bits that mma.sync gave; the call stays for programs that make the
- * choice. A synchronising call returns LSKUM_ERR_TIMEOUT if a wait inside a
+ * K 16 into tensor memory, all layers of 128 samples in one CTA); the call
+ * stays for programs that make the choice. A synchronising call returns LSKUM_ERR_TIMEOUT if a wait inside a
  * pass ran out (bounded waits: the kernel sets a flag and returns). */
 #define LSKUM_MLP_GEMM_MMA_SYNC 0
 #define LSKUM_MLP_GEMM_TCGEN05 1

@@ -1,16 +1,16 @@
 // The FP64 path's flux kernel for gamma = 1.4, its per-neighbour work in float
 // pairs (flux_pair.cuh).
 //
-// What bounds it: a split-flux difference costs 225 FP64 instructions per
-// neighbour entry, and the FP64 pipe issues two per clock and SM where the
-// FP32 pipes issue 128. The pair form takes about 1,500 FP32 instructions: at
-// 2.5M points 2.83 ms a launch instead of 14.75, at 0.6M 0.98 instead of 3.58
-// (a quarter of its entries are FP64 ones), at 5,120 0.070 instead of 0.148.
-// Entries that are not the pair form's (large steps, states out of its
-// range) are noted in a bit mask and evaluated in FP64 after the loop, with
-// the code of lskum_kernels.cu's k_flux, a warp's entries spread evenly over
-// its lanes; the stage update, the next stage's q-variables and the residue
-// stay FP64.
+// What bounds it: instruction issue (66 % of the slots at 2.5M points). A
+// split-flux difference costs 225 FP64 instructions per neighbour entry, and the
+// FP64 pipe issues two per clock and SM where the FP32 pipes issue 128. The pair
+// form takes about 1,850 FP32 instructions: at 2.5M points 2.89 ms a launch
+// instead of 14.75, at 0.6M 0.95 instead of 3.58, at 5,120 0.055 instead of
+// 0.148. Entries that are not the pair form's (large steps: a quarter at 0.6M,
+// most at 5,120) are noted in a bit mask and evaluated after the loop in 64-bit
+// fixed point (flux_fixed.cuh; by k_flux's FP64 formulas the launches took 0.99
+// and 0.068), a warp's entries spread evenly over its lanes; the stage update,
+// the next stage's q-variables and the residue stay FP64.
 
 #include "flux_fixed.cuh"
 #include "flux_fp64.cuh"
@@ -108,8 +108,8 @@ __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& 
     c[3] = fma(wn, dn[3], ws * ds[3]);
 }
 
-// The pair-form part of one point's entries first, first + stride, ...: adds to
-// acc; returns the entries left for FP64 as a bit mask.
+// The pair-form part of one point's entries first, first + kClasses, ...: adds to
+// acc; returns the entries left over as a bit mask.
 struct PairPoint {
     V4 q;
     DQP dq;
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
                                                      const DQP* __restrict__ dq,
                                                      V4* __restrict__ q_out) {
     static_assert(LANES == 1 || LANES == kClasses, "a thread takes all classes of a point or one");
-    // per warp: the FP64 entries of one round (owner lane, slot) and their results
+    // per warp: the large-step entries of one pass of its lanes (owner lane, slot) and their results
     __shared__ uint16_t s_item[BLOCK / 32][32];
     __shared__ double s_res[BLOCK / 32][4][32];
     __shared__ double s_R[LANES > 1 ? BLOCK / LANES : 1][4];
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
     const int8_t fl = live ? g.flag[d] : int8_t(LSKUM_INTERIOR);
     const bool fixed = ph.outer_fixed && fl == LSKUM_OUTER;
     const bool local = fl != LSKUM_INTERIOR;
-    uint32_t left = 0;  // entries for the FP64 evaluation
+    uint32_t left = 0;  // entries with large steps
     Pf acc[4] = {};
     if (live && !fixed) {
         PairPoint P;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
     double R[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) R[m] = double(acc[m].h) + double(acc[m].l);
-    // FP64 entries: the warp's lanes share them out evenly, 32 a round, and
+    // entries with large steps: the warp's lanes share them out evenly, 32 a time, and
     // each point adds its own class by class
     const int mine = __popc(left);
     int upto = mine;
