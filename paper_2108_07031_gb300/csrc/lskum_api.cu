@@ -353,7 +353,7 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
         if ((e = upload(c, &g.wx, L.wx)) != cudaSuccess || (e = upload(c, &g.wy, L.wy)) != cudaSuccess)
             return bail(e, "upload of the FP64 cloud layout");
         if (c->pairs) {
-            const float *half = nullptr, *weight = nullptr;
+            const HostLayout::Float4 *half = nullptr, *weight = nullptr;
             if ((e = upload(c, &half, L.half)) != cudaSuccess ||
                 (e = upload(c, &weight, L.weight)) != cudaSuccess)
                 return bail(e, "upload of the float-pair cloud layout");
@@ -365,12 +365,11 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
                    (e = upload(c, &g.wn, L.wn)) != cudaSuccess) {
             return bail(e, "upload of the FP64 cloud layout");
         }
-        std::vector<V4> lcoef(L.lc.size() / 4), lsum(L.lsum.size() / 4);
-        std::memcpy(lcoef.data(), L.lc.data(), L.lc.size() * sizeof(double));
-        std::memcpy(lsum.data(), L.lsum.data(), L.lsum.size() * sizeof(double));
-        if ((e = upload(c, &g.lcoef, lcoef)) != cudaSuccess ||
-            (e = upload(c, &g.lsum, lsum)) != cudaSuccess)
+        const double *lcoef = nullptr, *lsum = nullptr;
+        if ((e = upload(c, &lcoef, L.lc)) != cudaSuccess || (e = upload(c, &lsum, L.lsum)) != cudaSuccess)
             return bail(e, "upload of the FP64 inner-sweep coefficients");
+        g.lcoef = reinterpret_cast<const V4*>(lcoef);
+        g.lsum = reinterpret_cast<const V4*>(lsum);
     } else {
         // FP32 records per neighbour entry: {ws, wn, hdx, hdy} and {wx, wy};
         // per point the coordinates as float pairs (device order)

@@ -36,8 +36,11 @@ struct HostLayout {
     std::vector<double> wx, wy;    // full-stencil least-squares weights (Eq. 11)
     std::vector<double> ws, wn;    // split-stencil weights of d/ds and d/dn (Eq. 24)
     // with `pairs`, in place of hdx, hdy, ws, wn: {hdx hi, lo, hdy hi, lo} and
-    // {ws hi, lo, wn hi, lo}, four floats a slot
-    std::vector<float> half, weight;
+    // {ws hi, lo, wn hi, lo}
+    struct Float4 {
+        float v[4];
+    };
+    std::vector<Float4> half, weight;
     // FP64 inner sweeps (Eq. 29) split as q_x = (first-order q_x) - sum_j wx_j
     // (hdx_j (qx_j - qx_i) + hdy_j (qy_j - qy_i)), likewise q_y: per slot the
     // products {wx hdx, wx hdy, wy hdx, wy hdy} (4 per slot, [slot][stride]),

@@ -178,8 +178,8 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
     L.wx.assign(size_t(slots) * S, 0.0);
     L.wy.assign(size_t(slots) * S, 0.0);
     if (pairs) {
-        L.half.assign(size_t(slots) * S * 4, 0.0f);
-        L.weight.assign(size_t(slots) * S * 4, 0.0f);
+        L.half.assign(size_t(slots) * S, {});
+        L.weight.assign(size_t(slots) * S, {});
     } else {
         L.hdx.assign(size_t(slots) * S, 0.0);
         L.hdy.assign(size_t(slots) * S, 0.0);
@@ -290,8 +290,8 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
             L.wx[at] = wt[k] * (dx[k] * syy - dy[k] * sxy) / det;
             L.wy[at] = wt[k] * (dy[k] * sxx - dx[k] * sxy) / det;
             if (pairs) {
-                split2(hx, hy, &L.half[4 * at]);
-                split2(ws, wn, &L.weight[4 * at]);
+                split2(hx, hy, L.half[at].v);
+                split2(ws, wn, L.weight[at].v);
             } else {
                 L.hdx[at] = hx;
                 L.hdy[at] = hy;
