@@ -45,11 +45,13 @@ __device__ __forceinline__ Pf split_pair(const double x) {
 }
 #endif
 
-// The double equal to a float, by integer operations; subnormals give zero.
+// The double equal to a float, infinities and NaN included, by integer
+// operations; subnormals give zero.
 LSKUM_HD double widen(const float x) {
     const uint32_t u = fbits(x), mag = u & 0x7fffffffu;
     const bool zero = mag < 0x00800000u;
-    return dvalue(uint64_t((u & 0x80000000u) | (zero ? 0u : (mag >> 3) + 0x38000000u)) << 32 |
+    const uint32_t rebias = mag >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+    return dvalue(uint64_t((u & 0x80000000u) | (zero ? 0u : (mag >> 3) + rebias)) << 32 |
                   (zero ? 0u : u << 29));
 }
 
