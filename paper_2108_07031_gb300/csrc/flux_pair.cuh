@@ -46,6 +46,10 @@ constexpr Pf kTwentyFourth = {0x1.555556p-5f, -0x1.555556p-30f};
 constexpr Pf k120th = {0x1.111112p-7f, -0x1.dddddep-32f};
 constexpr float kPairMaxBeta = 16777216.0f, kPairMinBeta = 1.0f / 16777216.0f;
 
+// 2^-60 <= x < 2^60: with the low words and the products' errors in range too
+// (m1 lies between m0 and m3). False for NaN.
+LSKUM_HD bool pair_held(float x) { return fbits(x) - 0x21800000u < 0x3c000000u; }
+
 // exp(x) for |x| <= kPairMaxArg.
 LSKUM_HD Pf exp_pair(Pf x) {
     const float kf = rsub(rfma(x.h, kPairInvLn2N, 12582912.0f), 12582912.0f);
@@ -140,6 +144,8 @@ LSKUM_HD bool pair_state(const Pf b[4], const Pf d[4], PairState& w) {
     const Pf r1 = norm(add(add(r0, e), mul(r0, e)));
     const Pf r3 = norm(add(add(r1, e), mul(r1, e)));
     const Pf m0 = norm(mul(exp_pair(arg), mul(sq(i2), i2))), m1 = norm(mul(m0, i0)), m3 = mul(m1, i0);
+    // beta and ln E near their ends together: moments that floats do not hold
+    if (!(pair_held(m0.h) && pair_held(m3.h))) return false;
     w.dm0 = mul(m0, r0);
     w.dm1 = mul(m1, r1);
     w.dm3 = mul(m3, r3);
