@@ -76,7 +76,10 @@ int lskum_mlp_gradients(lskum_mlp* h, const float* feat_dev, const float* target
  * caller keeps feat_dev and target_dev unchanged until that stream has run
  * it (lskum_mlp_sync, or order its own writes after it by running on the
  * same stream, see lskum_mlp_set_stream). With loss non-NULL it returns
- * after the step. */
+ * after the step. A step of which a wait ran out, and steps queued after it, are
+ * not applied: parameters, moments and step count stay those of the last step
+ * before it. The next synchronising call returns LSKUM_ERR_TIMEOUT, and training
+ * can go on from there (lskum_mlp_set_params clears the failure too). */
 int lskum_mlp_train_step(lskum_mlp* h, const float* feat_dev, const float* target_dev, int64_t n,
                          float lr, double* loss);
 

@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/lskum_mlp.h"
@@ -38,6 +39,19 @@ struct LayerPtrs {
     int64_t b_off[kLayers];
     __nv_bfloat16* W[kLayers];
 };
+
+// Raised when a bounded wait of a pass runs out: the passes' bits on the device,
+// where the kernels that change the parameters read them, and 1 in pinned
+// memory, where the host looks after it has synchronised.
+enum Pass { kPassForward = 1, kPassBackward = 2, kPassWeightGrads = 4 };
+struct ErrFlag {
+    int* dev;
+    int* host;
+};
+__device__ __forceinline__ void raise(const ErrFlag f, Pass pass) {
+    atomicOr(f.dev, int(pass));
+    *f.host = 1;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return uint32_t(__cvta_generic_to_shared(p));
@@ -211,7 +225,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
 // feat: n x 32 FP32; Wp: the operand images (packed_offset); p: the FP32
 // parameters (biases; L's offsets), W5: the output layer's BF16 weights 4 x 256.
 // out: n x 4. TRAIN: also Af[l], Ab[l] of the hidden layers, and Ab[0], in granules.
-// *err receives 1 if a wait ran out (the outputs are then incomplete).
+// `err` is raised if a wait ran out (the outputs are then incomplete).
 struct FwdStore {
     float* Af[kLayers];
     __nv_bfloat16* Ab[kLayers];
@@ -221,7 +235,7 @@ template <bool TRAIN>
 __global__ void __launch_bounds__(kFwdThreads, 1)
     k_forward(const float* __restrict__ feat, int64_t n, const unsigned char* __restrict__ Wp,
               const float* __restrict__ p, LayerPtrs L, float* __restrict__ out, FwdStore st,
-              int* __restrict__ err) {
+              ErrFlag err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sA = smem_u32(smem), sRing = sA + kFwdOffRing;
@@ -401,7 +415,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             }
         }
     }
-    if (!ok && lane == 0) *err = 1;
+    if (!ok && lane == 0) raise(err, kPassForward);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     __syncwarp();
@@ -452,7 +466,7 @@ struct BwdArgs {
     double* sq;                    // [4 gridDim]
 };
 
-__global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, int64_t n, int* __restrict__ err) {
+__global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, int64_t n, ErrFlag err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sA = smem_u32(smem), sRing = sA + kFwdOffRing;
@@ -630,7 +644,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_backward(const BwdArgs a, in
             }
         }
     }
-    if (!ok && lane == 0) *err = 1;
+    if (!ok && lane == 0) raise(err, kPassBackward);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     __syncwarp();
@@ -663,7 +677,7 @@ constexpr int kDwSmem = kDwOffBar + 64;
 static_assert(kDwSmem <= 227 * 1024, "one CTA's shared memory");
 
 __global__ void __launch_bounds__(kDwThreads, 1) k_weight_grads(const DwArgs a, int n, int tiles_per_slice,
-                                                                int* __restrict__ err) {
+                                                                ErrFlag err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tiles = (n + kFwdRows - 1) / kFwdRows;
@@ -768,7 +782,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_weight_grads(const DwArgs a, 
             }
         }
     }
-    if (!ok && lane == 0) *err = 1;
+    if (!ok && lane == 0) raise(err, kPassWeightGrads);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     __syncwarp();
@@ -852,11 +866,14 @@ __global__ void k_features(const float* __restrict__ raw, int64_t n, const float
 }
 
 // Adam on the flat FP32 parameter vector; the BF16 copies are refreshed after it.
+// Nothing changes once a wait has run out in this step or one before it; *done
+// receives the number of an applied step.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
+                       float c1, float c2, const int* __restrict__ err, int64_t step, int64_t* done) {
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *err) return;
+    if (i == 0) *done = step;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -866,7 +883,8 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 }
 
 // BF16 copies of the weights: row-major, and as the operand images of the fused
-// forward and backward passes.
+// forward and backward passes. (Parameters that Adam left alone give the same
+// copies again.)
 __global__ void k_weights_bf16(const float* __restrict__ p, LayerPtrs L, unsigned char* __restrict__ Wp,
                                unsigned char* __restrict__ Wt) {
     const int l = blockIdx.y;
@@ -912,7 +930,8 @@ struct lskum_mlp {
     unsigned char* Wp = nullptr;  // operand images of the weights: forward pass
     unsigned char* Wt = nullptr;  // and backward pass
     int sms = 0;
-    int* err = nullptr;  // pinned: set by a forward pass one of whose waits ran out
+    ErrFlag err{};          // raised by a pass one of whose waits ran out
+    int64_t* done = nullptr;  // pinned: the last step that Adam applied
     std::vector<void*> allocs;
 };
 
@@ -943,12 +962,22 @@ inline unsigned blocks(int64_t n, int b) { return unsigned((n + b - 1) / b); }
 
 constexpr int kMaxSlices = 15;  // of ten blocks: one wave
 
-// After a synchronising call: LSKUM_ERR_TIMEOUT (and the flag cleared) if a
-// forward pass gave up one of its waits.
-int check_gemm_status(lskum_mlp* h) {
-    if (!*static_cast<volatile int*>(h->err)) return LSKUM_OK;
-    *h->err = 0;
-    return fail(LSKUM_ERR_TIMEOUT, "forward pass: a wait ran out");
+// After a synchronising call: LSKUM_ERR_TIMEOUT if a pass gave up one of its waits.
+// The steps queued from that pass on were not applied; they are not counted, and
+// with the flag cleared the handle goes on from the last applied one.
+int check_passes(lskum_mlp* h) {
+    if (!*static_cast<volatile int*>(h->err.host)) return LSKUM_OK;
+    int passes = 0;
+    MLP_CUDA(cudaMemcpyAsync(&passes, h->err.dev, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    MLP_CUDA(cudaMemsetAsync(h->err.dev, 0, sizeof(int), h->stream));
+    MLP_CUDA(cudaStreamSynchronize(h->stream));
+    *h->err.host = 0;
+    h->step = *static_cast<volatile int64_t*>(h->done);
+    std::string which;
+    for (const auto& [bit, name] : {std::pair(kPassForward, "forward pass"), std::pair(kPassBackward, "backward pass"),
+                                    std::pair(kPassWeightGrads, "weight gradients")})
+        if (passes & bit) which += std::string(which.empty() ? "" : ", ") + name;
+    return fail(LSKUM_ERR_TIMEOUT, which + ": a wait ran out");
 }
 
 // Forward pass from features (FP32 n x 32) to out (n x 4); train: the hidden
@@ -1044,7 +1073,8 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
     h->nparam = lskum_mlp_num_params();
     auto bail = [&](cudaError_t e) {
         for (void* p : h->allocs) cudaFree(p);
-        if (h->err) cudaFreeHost(h->err);
+        if (h->err.host) cudaFreeHost(h->err.host);
+        if (h->done) cudaFreeHost(h->done);
         if (h->own_stream) cudaStreamDestroy(h->own_stream);
         delete h;
         return fail(LSKUM_ERR_CUDA, std::string("lskum_mlp_create: ") + cudaGetErrorString(e));
@@ -1073,9 +1103,13 @@ int lskum_mlp_create(int64_t capacity, const float* proj, lskum_mlp** out) {
         (e = alloc(h, &h->Wt, packed_offset_t(0, 0, 0))) != cudaSuccess ||
         (e = alloc(h, &h->loss_dev, 1)) != cudaSuccess ||
         (e = alloc(h, &h->Wp, packed_offset(kLayers - 1, 0, 0))) != cudaSuccess ||
-        (e = cudaMallocHost(&h->err, sizeof(int))) != cudaSuccess)
+        (e = alloc(h, &h->err.dev, 1)) != cudaSuccess ||
+        (e = cudaMallocHost(&h->err.host, sizeof(int))) != cudaSuccess ||
+        (e = cudaMallocHost(&h->done, sizeof(int64_t))) != cudaSuccess ||
+        (e = cudaMemset(h->err.dev, 0, sizeof(int))) != cudaSuccess)
         return bail(e);
-    *h->err = 0;
+    *h->err.host = 0;
+    *h->done = 0;
     if ((e = cudaFuncSetAttribute(k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem)) !=
             cudaSuccess ||
         (e = cudaFuncSetAttribute(k_weight_grads, cudaFuncAttributeMaxDynamicSharedMemorySize, kDwSmem)) !=
@@ -1106,7 +1140,8 @@ void lskum_mlp_destroy(lskum_mlp* h) {
     if (!h) return;
     cudaStreamSynchronize(h->stream);
     for (void* p : h->allocs) cudaFree(p);
-    cudaFreeHost(h->err);
+    cudaFreeHost(h->err.host);
+    cudaFreeHost(h->done);
     cudaStreamDestroy(h->own_stream);
     delete h;
 }
@@ -1116,11 +1151,14 @@ int lskum_mlp_set_params(lskum_mlp* h, const float* params, int64_t n) {
     MLP_CUDA(cudaMemcpyAsync(h->p, params, sizeof(float) * n, cudaMemcpyHostToDevice, h->stream));
     MLP_CUDA(cudaMemsetAsync(h->m, 0, sizeof(float) * n, h->stream));
     MLP_CUDA(cudaMemsetAsync(h->v, 0, sizeof(float) * n, h->stream));
-    h->step = 0;
+    MLP_CUDA(cudaMemsetAsync(h->err.dev, 0, sizeof(int), h->stream));  // new parameters: earlier steps no longer count
     MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L,
                                                                                                       h->Wp, h->Wt),
               cudaGetLastError()));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
+    *h->err.host = 0;
+    *h->done = 0;
+    h->step = 0;
     return LSKUM_OK;
 }
 
@@ -1149,7 +1187,7 @@ int lskum_mlp_predict(lskum_mlp* h, const float* feat, int64_t n, float* out) {
     if (to != out)
         MLP_CUDA(cudaMemcpyAsync(out, to, sizeof(float) * n * kOut, cudaMemcpyDeviceToDevice, h->stream));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
-    return check_gemm_status(h);
+    return check_passes(h);
 }
 
 int lskum_mlp_gradients(lskum_mlp* h, const float* feat, const float* target, int64_t n, float* grads,
@@ -1164,7 +1202,7 @@ int lskum_mlp_gradients(lskum_mlp* h, const float* feat, const float* target, in
     if (grads) MLP_CUDA(cudaMemcpyAsync(grads, h->g, sizeof(float) * h->nparam, cudaMemcpyDeviceToHost, h->stream));
     if (loss) MLP_CUDA(cudaMemcpyAsync(loss, h->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     MLP_CUDA(cudaStreamSynchronize(h->stream));
-    return check_gemm_status(h);
+    return check_passes(h);
 }
 
 int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, int64_t n, float lr,
@@ -1181,7 +1219,7 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, i
     const float c1 = 1.f / (1.f - powf(b1, float(h->step)));
     const float c2 = 1.f / (1.f - powf(b2, float(h->step)));
     MLP_CUDA((k_adam<<<blocks(h->nparam, 256), 256, 0, h->stream>>>(h->p, h->g, h->m, h->v, h->nparam, lr, b1, b2,
-                                                                     1e-8f, c1, c2),
+                                                                     1e-8f, c1, c2, h->err.dev, h->step, h->done),
               cudaGetLastError()));
     MLP_CUDA((k_weights_bf16<<<dim3(blocks(int64_t(kWidth) * kWidth, 256), kLayers), 256, 0, h->stream>>>(h->p, h->L,
                                                                                                       h->Wp, h->Wt),
@@ -1189,7 +1227,7 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, i
     if (loss) {
         MLP_CUDA(cudaMemcpyAsync(loss, h->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         MLP_CUDA(cudaStreamSynchronize(h->stream));
-        return check_gemm_status(h);
+        return check_passes(h);
     }
     return LSKUM_OK;
 }
@@ -1197,7 +1235,7 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat, const float* target, i
 int lskum_mlp_sync(lskum_mlp* h) {
     if (!h) return fail(LSKUM_ERR_INVALID_ARG, "null");
     MLP_CUDA(cudaStreamSynchronize(h->stream));
-    return check_gemm_status(h);
+    return check_passes(h);
 }
 
 int lskum_mlp_set_gemm(lskum_mlp* h, int path) {
