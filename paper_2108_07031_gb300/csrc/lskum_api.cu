@@ -47,7 +47,7 @@ struct lskum_ctx {
 
     HostLayout host;
     bool mixed = false;
-    bool pairs = false;  // FP64 path: the fused flux in float pairs (gamma = 1.4)
+    bool pairs = false;  // FP64 path: the fused flux in float pairs (gamma = 1.4, HostLayout::held)
     DevGeom g{};
     DevGeomPair gp{};
     DevGeom32 g32{};
@@ -146,15 +146,22 @@ int n_blocks(const lskum_ctx* c) {
     return int((c->g.n + c->block - 1) / c->block);
 }
 
+// Where the last sweep leaves the derivatives as float pairs for the pair-form
+// flux: the dq buffer that it does not gather from or write to.
+DQP* pair_buffer(const lskum_ctx* c) {
+    const int inner = c->opt.inner_iters;
+    return reinterpret_cast<DQP*>(c->st.dq[inner == 0 ? 1 : inner == 1 ? 2 : 0]);
+}
+
 // q-derivatives of the q buffer `qb` into dq[final] (FP64; for_flux: in float
-// pairs if the flux kernel takes them so) or dq32[final] (mixed); returns the
+// pairs too if the flux kernel takes them) or dq32[final] (mixed); returns the
 // index of the buffer holding the result.
 cudaError_t run_q_derivatives(lskum_ctx* c, int qb, bool for_flux, int* final_buf, int64_t* launches) {
-    const bool pairs = for_flux && c->pairs;
+    DQP* const pairs = for_flux && c->pairs ? pair_buffer(c) : nullptr;
     cudaError_t e = timed(c, kLsFirst, [&] {
         return c->mixed ? launch_ls_first_mx(c->g, c->g32, c->st.qhl[qb], c->st.dq32[0], c->block_ls, c->stream)
-                        : launch_ls_first(c->g, c->st.q[qb], c->st.dq[0], pairs && c->opt.inner_iters == 0,
-                                          c->block_ls, c->stream);
+                        : launch_ls_first(c->g, c->st.q[qb], c->st.dq[0],
+                                          c->opt.inner_iters == 0 ? pairs : nullptr, c->block_ls, c->stream);
     });
     if (e != cudaSuccess) return e;
     ++*launches;
@@ -167,7 +174,7 @@ cudaError_t run_q_derivatives(lskum_ctx* c, int qb, bool for_flux, int* final_bu
             return c->mixed ? launch_ls_inner_mx(c->g, c->g32, c->st.dq32[0], c->st.dq32[cur],
                                                  c->st.dq32[next], c->block_ls, c->stream)
                             : launch_ls_inner(c->g, c->st.dq[0], c->st.dq[cur], c->st.dq[next],
-                                              pairs && it + 1 == c->opt.inner_iters, c->block_ls,
+                                              it + 1 == c->opt.inner_iters ? pairs : nullptr, c->block_ls,
                                               c->stream);
         });
         if (e != cudaSuccess) return e;
@@ -186,8 +193,7 @@ cudaError_t launch_flux_any(lskum_ctx* c, int mode, int qb, int dbuf, int qout) 
         return launch_flux_split(mode, c->g, c->ph, c->st, c->st.q[qb], c->st.dq[dbuf],
                                  qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
     if (c->pairs)
-        return launch_flux_pair(mode, c->g, c->gp, c->ph, c->st, c->st.q[qb],
-                                reinterpret_cast<const DQP*>(c->st.dq[dbuf]),
+        return launch_flux_pair(mode, c->g, c->gp, c->ph, c->st, c->st.q[qb], c->st.dq[dbuf], pair_buffer(c),
                                 qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
     return launch_flux(mode, c->g, c->ph, c->st, c->st.q[qb], c->st.dq[dbuf],
                        qout >= 0 ? c->st.q[qout] : nullptr, c->block, c->stream);
@@ -304,6 +310,11 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
     // host validation and layout first: input errors are reported without a GPU
     std::string err;
     int rc = build_layout(n, xy, normals, flags, nbr_offsets, nbr_idx, o, c->pairs, c->host, err);
+    if (rc == LSKUM_OK && c->pairs && !c->host.held) {  // sizes the pair kernel does not take: FP64 throughout
+        c->pairs = false;
+        c->host = HostLayout();
+        rc = build_layout(n, xy, normals, flags, nbr_offsets, nbr_idx, o, false, c->host, err);
+    }
     if (rc != LSKUM_OK) {
         delete c;
         return fail(rc, err);
@@ -354,9 +365,11 @@ int lskum_create(int64_t n, const double* xy, const double* normals, const int8_
             return bail(e, "upload of the FP64 cloud layout");
         if (c->pairs) {
             const HostLayout::Float4 *half = nullptr, *weight = nullptr;
+            const HostLayout::Rest4* rest = nullptr;
             if ((e = upload(c, &half, L.half)) != cudaSuccess ||
-                (e = upload(c, &weight, L.weight)) != cudaSuccess)
+                (e = upload(c, &weight, L.weight)) != cudaSuccess || (e = upload(c, &rest, L.rest)) != cudaSuccess)
                 return bail(e, "upload of the float-pair cloud layout");
+            c->gp.rest = reinterpret_cast<const char4*>(rest);
             c->gp.half = reinterpret_cast<const float4*>(half);
             c->gp.weight = reinterpret_cast<const float4*>(weight);
         } else if ((e = upload(c, &g.hdx, L.hdx)) != cudaSuccess ||

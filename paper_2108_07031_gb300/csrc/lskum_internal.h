@@ -35,12 +35,20 @@ struct HostLayout {
     std::vector<double> hdx, hdy;  // half of the global offsets x_j - x_i, y_j - y_i
     std::vector<double> wx, wy;    // full-stencil least-squares weights (Eq. 11)
     std::vector<double> ws, wn;    // split-stencil weights of d/ds and d/dn (Eq. 24)
-    // with `pairs`, in place of hdx, hdy, ws, wn: {hdx hi, lo, hdy hi, lo} and
-    // {ws hi, lo, wn hi, lo}
+    // with `pairs`, in place of hdx, hdy, ws, wn: {hdx hi, lo, hdy hi, lo},
+    // {ws hi, lo, wn hi, lo} and, a byte each, by how many units in the last place
+    // of the double the four exceed their hi + lo. held: all of them are of a size
+    // that this holds and the pair kernel computes with (else the layout is to be
+    // built without `pairs`).
     struct Float4 {
         float v[4];
     };
+    struct Rest4 {
+        int8_t v[4];
+    };
     std::vector<Float4> half, weight;
+    std::vector<Rest4> rest;
+    bool held = true;
     // FP64 inner sweeps (Eq. 29) split as q_x = (first-order q_x) - sum_j wx_j
     // (hdx_j (qx_j - qx_i) + hdy_j (qy_j - qy_i)), likewise q_y: per slot the
     // products {wx hdx, wx hdy, wy hdx, wy hdy} (4 per slot, [slot][stride]),

@@ -40,26 +40,25 @@ namespace {
 // inner one; at 0.6M points and more both forms are bound by the FP64 pipe
 // (190 and 285 us). A component's sum keeps the slot order.
 
-// Stores a component's derivatives: FP64, or as float pairs for the pair-form
-// flux kernel (hi and lo each rounded to nearest).
+// Stores a component's derivatives, with PAIRS also as float pairs (hi and lo each
+// rounded to nearest) for the pair-form flux kernel.
 template <bool PAIRS>
-__device__ __forceinline__ void store_dq(V8* p, const int m, const double x, const double y) {
+__device__ __forceinline__ void store_dq(V8* p, DQP* pairs, const int m, const double x, const double y) {
+    p->x[m] = x;
+    p->y[m] = y;
     if (PAIRS) {
         float4 v;
         v.x = __double2float_rn(x);
         v.y = __double2float_rn(x - double(v.x));
         v.z = __double2float_rn(y);
         v.w = __double2float_rn(y - double(v.z));
-        reinterpret_cast<DQP*>(p)->c[m] = v;
-    } else {
-        p->x[m] = x;
-        p->y[m] = y;
+        pairs->c[m] = v;
     }
 }
 
 template <int BLOCK, bool PAIRS>
 __global__ void __launch_bounds__(BLOCK) k_ls_first(const DevGeom g, const V4* __restrict__ q,
-                                                    V8* __restrict__ dq) {
+                                                    V8* __restrict__ dq, DQP* __restrict__ pairs) {
     const int64_t t = (int64_t(blockIdx.x) * BLOCK + threadIdx.x) / 4;  // (point, condition)
     const int m = threadIdx.x % 4;
     const int64_t d = t >> g.cshift;
@@ -78,7 +77,7 @@ __global__ void __launch_bounds__(BLOCK) k_ls_first(const DevGeom g, const V4* _
         ax += wx * e;
         ay += wy * e;
     }
-    store_dq<PAIRS>(dq + t, m, ax, ay);
+    store_dq<PAIRS>(dq + t, pairs + t, m, ax, ay);
 }
 
 // One Jacobi sweep of Eq. 29. With dq~_j = (q_j - q_i) - (hdx_j (qx_j - qx_i)
@@ -89,11 +88,12 @@ __global__ void __launch_bounds__(BLOCK) k_ls_first(const DevGeom g, const V4* _
 // the same stage (dq_first), so a sweep gathers only the neighbours'
 // derivatives: 4 FMAs per component and neighbour instead of 7 FP64
 // operations. The bracket is ~1e-4 of q_x at 10M points and is formed to
-// ~1e-12 of itself, so q_x keeps FP64 accuracy.
+// ~1e-12 of itself, so q_x keeps FP64 accuracy. `pairs` may be the memory of
+// dq_first: a record is read by its own four threads only, before they write it.
 template <int BLOCK, bool PAIRS>
-__global__ void __launch_bounds__(BLOCK) k_ls_inner(const DevGeom g, const V8* __restrict__ dq_first,
+__global__ void __launch_bounds__(BLOCK) k_ls_inner(const DevGeom g, const V8* dq_first,
                                                     const V8* __restrict__ din,
-                                                    V8* __restrict__ dout) {
+                                                    V8* __restrict__ dout, DQP* pairs) {
     const int64_t t = (int64_t(blockIdx.x) * BLOCK + threadIdx.x) / 4;  // (point, condition)
     const int m = threadIdx.x % 4;
     const int64_t d = t >> g.cshift;
@@ -113,14 +113,16 @@ __global__ void __launch_bounds__(BLOCK) k_ls_inner(const DevGeom g, const V8* _
     }
     const V4 S = g.lsum[d];
     const double xi = din[t].x[m], yi = din[t].y[m];
-    store_dq<PAIRS>(dout + t, m, dq_first[t].x[m] - (ax - fma(S.a, xi, S.b * yi)),
-                    dq_first[t].y[m] - (ay - fma(S.c, xi, S.d * yi)));
+    const double fx = dq_first[t].x[m], fy = dq_first[t].y[m];
+    if (PAIRS) __syncwarp(0xfu << (threadIdx.x & 28));
+    store_dq<PAIRS>(dout + t, pairs + t, m, fx - (ax - fma(S.a, xi, S.b * yi)), fy - (ay - fma(S.c, xi, S.d * yi)));
 }
 
 // ------------------------------------------------------- flux residual + RK
 
-// Every gamma but 1.4, which k_flux_pair takes.
-template <int MODE, int BLOCK>
+// Every gamma but 1.4, and 1.4 on clouds of sizes that k_flux_pair does not take
+// (HostLayout::held).
+template <int MODE, int BLOCK, bool G14>
 __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics ph,
                                                 const DevState st, const V4* __restrict__ q_in,
                                                 const V8* __restrict__ dq, V4* __restrict__ q_out) {
@@ -162,8 +164,8 @@ __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics p
                 if (!modified_states(second, second ? g.hdx[at] : 0.0, second ? g.hdy[at] : 0.0,
                                      second ? dq[jt] : di, di, tj, t0))
                     continue;
-                Prim wj = q_to_prim<false>(tj[0], tj[1], tj[2], tj[3], ph.gm1_inv);
-                Prim w0 = q_to_prim<false>(t0[0], t0[1], t0[2], t0[3], ph.gm1_inv);
+                Prim wj = q_to_prim<G14>(tj[0], tj[1], tj[2], tj[3], ph.gm1_inv);
+                Prim w0 = q_to_prim<G14>(t0[0], t0[1], t0[2], t0[3], ph.gm1_inv);
                 if (local) {  // velocities into (s, n)
                     const double sj = wj.u * tx + wj.v * ty, nj = wj.u * nx + wj.v * ny;
                     const double s0 = w0.u * tx + w0.v * ty, n0 = w0.u * nx + w0.v * ny;
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux(const DevGeom g, const Physics p
                 R[2] = rs * ty + rn * ny;
             }
         }
-        r2 = stage_epilogue<MODE, false>(g, ph, st, t, d, fl, fixed, R, q_out);
+        r2 = stage_epilogue<MODE, G14>(g, ph, st, t, d, fl, fixed, R, q_out);
     }
     if (MODE == 1) {
         if (g.cshift == 0) {  // one condition: fused block partial sums
@@ -520,49 +522,56 @@ inline unsigned grid_nc(const DevGeom& g, int block) { return grid_for(g.n << g.
 
 }  // namespace
 
-cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, bool as_pairs, int block,
+cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, DQP* pairs, int block,
                             cudaStream_t s) {
     const unsigned grid = grid_for((g.n << g.cshift) * 4, block);
     if (block == 256) {
-        if (as_pairs) k_ls_first<256, true><<<grid, 256, 0, s>>>(g, q, dq);
-        else k_ls_first<256, false><<<grid, 256, 0, s>>>(g, q, dq);
+        if (pairs) k_ls_first<256, true><<<grid, 256, 0, s>>>(g, q, dq, pairs);
+        else k_ls_first<256, false><<<grid, 256, 0, s>>>(g, q, dq, nullptr);
     } else {
-        if (as_pairs) k_ls_first<kDefaultBlock, true><<<grid, kDefaultBlock, 0, s>>>(g, q, dq);
-        else k_ls_first<kDefaultBlock, false><<<grid, kDefaultBlock, 0, s>>>(g, q, dq);
+        if (pairs) k_ls_first<kDefaultBlock, true><<<grid, kDefaultBlock, 0, s>>>(g, q, dq, pairs);
+        else k_ls_first<kDefaultBlock, false><<<grid, kDefaultBlock, 0, s>>>(g, q, dq, nullptr);
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* din, V8* dout, bool as_pairs,
+cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* din, V8* dout, DQP* pairs,
                             int block, cudaStream_t s) {
     const unsigned grid = grid_for((g.n << g.cshift) * 4, block);
     if (block == 256) {
-        if (as_pairs) k_ls_inner<256, true><<<grid, 256, 0, s>>>(g, dq_first, din, dout);
-        else k_ls_inner<256, false><<<grid, 256, 0, s>>>(g, dq_first, din, dout);
+        if (pairs) k_ls_inner<256, true><<<grid, 256, 0, s>>>(g, dq_first, din, dout, pairs);
+        else k_ls_inner<256, false><<<grid, 256, 0, s>>>(g, dq_first, din, dout, nullptr);
     } else {
-        if (as_pairs) k_ls_inner<kDefaultBlock, true><<<grid, kDefaultBlock, 0, s>>>(g, dq_first, din, dout);
-        else k_ls_inner<kDefaultBlock, false><<<grid, kDefaultBlock, 0, s>>>(g, dq_first, din, dout);
+        if (pairs) k_ls_inner<kDefaultBlock, true><<<grid, kDefaultBlock, 0, s>>>(g, dq_first, din, dout, pairs);
+        else k_ls_inner<kDefaultBlock, false><<<grid, kDefaultBlock, 0, s>>>(g, dq_first, din, dout, nullptr);
     }
     return cudaGetLastError();
 }
 
-template <int BLOCK>
+template <int BLOCK, bool G14>
 static void flux_dispatch(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                           const V4* q_in, const V8* dq, V4* q_out, cudaStream_t s) {
     const unsigned grid = grid_nc(g, BLOCK);
     switch (mode) {
-        case 0: k_flux<0, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 1: k_flux<1, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 2: k_flux<2, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        case 3: k_flux<3, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
-        default: k_flux<4, BLOCK><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 0: k_flux<0, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 1: k_flux<1, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 2: k_flux<2, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        case 3: k_flux<3, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
+        default: k_flux<4, BLOCK, G14><<<grid, BLOCK, 0, s>>>(g, ph, st, q_in, dq, q_out); break;
     }
 }
 
 cudaError_t launch_flux(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                         const V4* q_in, const V8* dq, V4* q_out, int block, cudaStream_t s) {
-    if (block == 256) flux_dispatch<256>(mode, g, ph, st, q_in, dq, q_out, s);
-    else flux_dispatch<kDefaultBlock>(mode, g, ph, st, q_in, dq, q_out, s);
+    // gamma = 1.4: log-free density (see q_to_prim)
+    const bool g14 = fabs(ph.gm1_inv - 2.5) < 1e-12;
+    if (block == 256) {
+        if (g14) flux_dispatch<256, true>(mode, g, ph, st, q_in, dq, q_out, s);
+        else flux_dispatch<256, false>(mode, g, ph, st, q_in, dq, q_out, s);
+    } else {
+        if (g14) flux_dispatch<kDefaultBlock, true>(mode, g, ph, st, q_in, dq, q_out, s);
+        else flux_dispatch<kDefaultBlock, false>(mode, g, ph, st, q_in, dq, q_out, s);
+    }
     return cudaGetLastError();
 }
 

@@ -32,17 +32,19 @@ struct __align__(32) D8f {
 };
 
 // q-derivatives of one point as float pairs (hi + lo = the FP64 value to
-// ~2^-49), the flux kernel's input in the pair form: per component {q_x hi, lo,
+// ~2^-49), what the flux kernel's pair form reads: per component {q_x hi, lo,
 // q_y hi, lo}. The size of a V8.
 struct __align__(64) DQP {
     float4 c[4];
 };
 
 // Per-neighbour constants of the pair-form flux kernel, slot-major
-// [slot][stride], hi and lo floats interleaved.
+// [slot][stride], hi and lo floats interleaved; with `rest` the doubles themselves
+// (4 bytes an entry instead of 32 for a second copy).
 struct DevGeomPair {
     const float4* half;    // half offsets {hdx hi, lo, hdy hi, lo}
     const float4* weight;  // split-stencil weights {ws hi, lo, wn hi, lo}
+    const char4* rest;     // hdx, hdy, ws, wn less hi + lo, in units of their last place
 };
 
 // FP32 copies of the slot-major per-neighbour arrays (mixed precision).
@@ -136,19 +138,20 @@ __host__ __device__ __forceinline__ int64_t sidx(const DevGeom& g, int64_t d, ui
 }
 
 // Launchers (return cudaGetLastError()).
-// as_pairs: the result is written as DQP records (for launch_flux_pair)
-// instead of V8 ones, into the same memory.
-cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, bool as_pairs, int block,
+// pairs: the result also goes there as DQP records (for launch_flux_pair), unless
+// null. An inner sweep's may be dq_first's own memory when that is not dq_in.
+cudaError_t launch_ls_first(const DevGeom& g, const V4* q, V8* dq, DQP* pairs, int block,
                             cudaStream_t s);
 cudaError_t launch_ls_inner(const DevGeom& g, const V8* dq_first, const V8* dq_in, V8* dq_out,
-                            bool as_pairs, int block, cudaStream_t s);
+                            DQP* pairs, int block, cudaStream_t s);
 // mode 0: evaluate R only (written to st.R); mode 1..4: SSP-RK stage.
 cudaError_t launch_flux(int mode, const DevGeom& g, const Physics& ph, const DevState& st,
                         const V4* q_in, const V8* dq, V4* q_out, int block, cudaStream_t s);
-// The same for gamma = 1.4 with the neighbour pairs' work in float pairs.
+// The same for gamma = 1.4 with the neighbour pairs' work in float pairs (dqp) or,
+// where steps are large, in fixed point (dq).
 cudaError_t launch_flux_pair(int mode, const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
-                             const DevState& st, const V4* q_in, const DQP* dq, V4* q_out, int block,
-                             cudaStream_t s);
+                             const DevState& st, const V4* q_in, const V8* dq, const DQP* dqp, V4* q_out,
+                             int block, cudaStream_t s);
 // Threads it gives a point, and its blocks (of `block` threads) for the cloud.
 int pair_flux_lanes(const DevGeom& g);
 int64_t pair_flux_blocks(const DevGeom& g, int block);

@@ -30,7 +30,11 @@ constexpr int kClasses = 4;
 // 232 / 170, 150,598 429 / 403, 321,438 638 / 684, 600,138 960 / 1,091.
 constexpr int64_t kSplitPairs = 1 << 18;
 
-__device__ __forceinline__ double join(const Pf a) { return widen(a.h) + widen(a.l); }
+// The double of which h + l is the pair and r what it exceeds them by, in units of
+// its last place (lskum_setup.cpp); h and l are finite.
+__device__ __forceinline__ double whole(const float h, const float l, const signed char r) {
+    return bitsd(dbits(widen(h) + widen(l)) + r);
+}
 
 __device__ __forceinline__ Pf dx_of(const float4& c) { return Pf{c.x, c.y}; }
 __device__ __forceinline__ Pf dy_of(const float4& c) { return Pf{c.z, c.w}; }
@@ -58,7 +62,7 @@ __device__ __noinline__ void general_diff(const double* tj, const double* t0, co
 // what k_flux adds for that entry. 64 FP64 instructions and some 1,700 on the
 // integer pipe (flux_fixed.cuh), where k_flux's formulas take 230 FP64 ones.
 __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
-                                           const V4* __restrict__ q_in, const DQP* __restrict__ dq,
+                                           const V4* __restrict__ q_in, const V8* __restrict__ dq,
                                            const int64_t t, const int k, double c[4]) {
     const int64_t d = t >> g.cshift;
     const int64_t at = int64_t(k) * g.stride + d;
@@ -68,23 +72,15 @@ __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& 
     double tj[4] = {qj.a, qj.b, qj.c, qj.d};
     double t0[4] = {qi.a, qi.b, qi.c, qi.d};
     c[0] = c[1] = c[2] = c[3] = 0.0;
-    V8 vi, vj;
+    const char4 rest = gp.rest[at];
     double hx = 0.0, hy = 0.0;
     const bool second = ph.order == 2;
     if (second) {
         const float4 hp = gp.half[at];
-        const DQP di = dq[t], dj = dq[jt];
-        hx = join(Pf{hp.x, hp.y});
-        hy = join(Pf{hp.z, hp.w});
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            vi.x[m] = join(dx_of(di.c[m]));
-            vi.y[m] = join(dy_of(di.c[m]));
-            vj.x[m] = join(dx_of(dj.c[m]));
-            vj.y[m] = join(dy_of(dj.c[m]));
-        }
+        hx = whole(hp.x, hp.y, rest.x);
+        hy = whole(hp.z, hp.w, rest.y);
     }
-    if (!modified_states(second, hx, hy, vj, vi, tj, t0)) return;
+    if (!modified_states(second, hx, hy, dq[second ? jt : t], dq[t], tj, t0)) return;
     const uint32_t sc = e >> kIndexBits & 3u, nc = e >> (kIndexBits + 2) & 3u;
     const bool local = g.flag[d] != LSKUM_INTERIOR;
     const double2 nn = local ? g.nrm[d] : make_double2(0.0, 1.0);
@@ -101,7 +97,7 @@ __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& 
     }
     const float4 wp = gp.weight[at];
     // an entry outside a stencil has weight 0 there
-    const double ws = join(Pf{wp.x, wp.y}), wn = join(Pf{wp.z, wp.w});
+    const double ws = whole(wp.x, wp.y, rest.z), wn = whole(wp.z, wp.w, rest.w);
     c[0] = fma(wn, dn[0], ws * ds[0]);
     c[1] = fma(wn, dn[2], ws * ds[1]);
     c[2] = fma(wn, dn[1], ws * ds[2]);
@@ -203,7 +199,8 @@ template <int MODE, int BLOCK, int LANES>
 __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevGeomPair gp,
                                                      const Physics ph, const DevState st,
                                                      const V4* __restrict__ q_in,
-                                                     const DQP* __restrict__ dq,
+                                                     const V8* __restrict__ dq,
+                                                     const DQP* __restrict__ dqp,
                                                      V4* __restrict__ q_out) {
     static_assert(LANES == 1 || LANES == kClasses, "a thread takes all classes of a point or one");
     // per warp: the large-step entries of one pass of its lanes (owner lane, slot) and their results
@@ -224,7 +221,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
     if (live && !fixed) {
         PairPoint P;
         P.q = ld4(q_in + t);
-        P.dq = dq[t];
+        P.dq = dqp[t];
         P.local = local;
         const double2 nn = local ? g.nrm[d] : make_double2(0.0, 1.0);
         P.nx = split_pair(nn.x);
@@ -238,7 +235,7 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
 #pragma unroll 1
         for (int r = part; r < kClasses; r += LANES) {
             Pf sum[4] = {};
-            left |= entries_pair(g, gp, second, q_in, dq, d, cc, P, r, c, sum);
+            left |= entries_pair(g, gp, second, q_in, dqp, d, cc, P, r, c, sum);
 #pragma unroll
             for (int m = 0; m < 4; ++m) acc[m] = LANES == 1 ? add(acc[m], sum[m]) : sum[m];
         }
@@ -337,14 +334,15 @@ inline unsigned pair_grid(const DevGeom& g, int block, int lanes) {
 
 template <int BLOCK, int LANES>
 void pair_dispatch(int mode, const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
-                   const DevState& st, const V4* q_in, const DQP* dq, V4* q_out, cudaStream_t s) {
+                   const DevState& st, const V4* q_in, const V8* dq, const DQP* dqp, V4* q_out,
+                   cudaStream_t s) {
     const unsigned grid = pair_grid(g, BLOCK, LANES);
     switch (mode) {
-        case 0: k_flux_pair<0, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, q_out); break;
-        case 1: k_flux_pair<1, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, q_out); break;
-        case 2: k_flux_pair<2, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, q_out); break;
-        case 3: k_flux_pair<3, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, q_out); break;
-        default: k_flux_pair<4, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, q_out); break;
+        case 0: k_flux_pair<0, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, dqp, q_out); break;
+        case 1: k_flux_pair<1, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, dqp, q_out); break;
+        case 2: k_flux_pair<2, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, dqp, q_out); break;
+        case 3: k_flux_pair<3, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, dqp, q_out); break;
+        default: k_flux_pair<4, BLOCK, LANES><<<grid, BLOCK, 0, s>>>(g, gp, ph, st, q_in, dq, dqp, q_out); break;
     }
 }
 
@@ -359,15 +357,15 @@ int64_t pair_flux_blocks(const DevGeom& g, int block) {
 }
 
 cudaError_t launch_flux_pair(int mode, const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
-                             const DevState& st, const V4* q_in, const DQP* dq, V4* q_out, int block,
-                             cudaStream_t s) {
+                             const DevState& st, const V4* q_in, const V8* dq, const DQP* dqp, V4* q_out,
+                             int block, cudaStream_t s) {
     const bool split = pair_flux_lanes(g) > 1;
     if (block == 256) {
-        if (split) pair_dispatch<256, kClasses>(mode, g, gp, ph, st, q_in, dq, q_out, s);
-        else pair_dispatch<256, 1>(mode, g, gp, ph, st, q_in, dq, q_out, s);
+        if (split) pair_dispatch<256, kClasses>(mode, g, gp, ph, st, q_in, dq, dqp, q_out, s);
+        else pair_dispatch<256, 1>(mode, g, gp, ph, st, q_in, dq, dqp, q_out, s);
     } else {
-        if (split) pair_dispatch<kDefaultBlock, kClasses>(mode, g, gp, ph, st, q_in, dq, q_out, s);
-        else pair_dispatch<kDefaultBlock, 1>(mode, g, gp, ph, st, q_in, dq, q_out, s);
+        if (split) pair_dispatch<kDefaultBlock, kClasses>(mode, g, gp, ph, st, q_in, dq, dqp, q_out, s);
+        else pair_dispatch<kDefaultBlock, 1>(mode, g, gp, ph, st, q_in, dq, dqp, q_out, s);
     }
     return cudaGetLastError();
 }

@@ -63,13 +63,26 @@ inline Frame frame_of(int8_t flag, const double* nrm) {
     return {nrm[1], -nrm[0], nrm[0], nrm[1]};
 }
 
-// Two doubles as float pairs {a hi, a lo, b hi, b lo}.
-inline void split2(double a, double b, float* out) {
-    out[0] = float(a);
-    out[1] = float(a - double(out[0]));
-    out[2] = float(b);
-    out[3] = float(b - double(out[2]));
+// A double as a float pair {hi, lo}, with the units in its last place by which it
+// exceeds their sum in *rest (a pair holds 49 of the 53 bits, so a few). False if
+// that is not exact: a low word below the floats' range takes up to 2^-149,
+// nothing next to offsets and weights of the sizes below.
+inline bool split(double x, float* out, int8_t* rest) {
+    out[0] = float(x);
+    out[1] = float(x - double(out[0]));
+    const double sum = double(out[0]) + double(out[1]);
+    int64_t bx, bs;
+    std::memcpy(&bx, &x, 8);
+    std::memcpy(&bs, &sum, 8);
+    const int64_t r = bx - bs;
+    const bool exact = r >= -127 && r <= 127;
+    *rest = exact ? int8_t(r) : int8_t(0);
+    return exact || std::fabs(x - sum) <= 0x1p-140;
 }
+
+// The sizes of half offsets (the longer component) and weights that the pair
+// kernel takes: its products keep clear of the floats' ends.
+constexpr double kHeldLeast = 0x1p-30, kHeldMost = 0x1p30, kHeldWeight = 0x1p60;
 
 }  // namespace
 
@@ -180,6 +193,7 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
     if (pairs) {
         L.half.assign(size_t(slots) * S, {});
         L.weight.assign(size_t(slots) * S, {});
+        L.rest.assign(size_t(slots) * S, {});
     } else {
         L.hdx.assign(size_t(slots) * S, 0.0);
         L.hdy.assign(size_t(slots) * S, 0.0);
@@ -194,7 +208,8 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
 
     int64_t bad_point = -1;
     const char* bad_what = "";
-#pragma omp parallel for schedule(dynamic, 1024)
+    bool held = true;
+#pragma omp parallel for schedule(dynamic, 1024) reduction(&& : held)
     for (int64_t d = 0; d < n; ++d) {
         const int64_t i = L.dev_to_user[d];
         const int8_t fl = flags[i];
@@ -290,8 +305,14 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
             L.wx[at] = wt[k] * (dx[k] * syy - dy[k] * sxy) / det;
             L.wy[at] = wt[k] * (dy[k] * sxx - dx[k] * sxy) / det;
             if (pairs) {
-                split2(hx, hy, L.half[at].v);
-                split2(ws, wn, L.weight[at].v);
+                float *h = L.half[at].v, *w = L.weight[at].v;
+                int8_t* r = L.rest[at].v;
+                const double size = std::max(std::fabs(hx), std::fabs(hy));
+                const bool ok = split(hx, h, r) & split(hy, h + 2, r + 1) & split(ws, w, r + 2) &
+                                split(wn, w + 2, r + 3);
+                if (!(ok && size >= kHeldLeast && size <= kHeldMost && std::fabs(ws) <= kHeldWeight &&
+                      std::fabs(wn) <= kHeldWeight))
+                    held = false;
             } else {
                 L.hdx[at] = hx;
                 L.hdy[at] = hy;
@@ -308,6 +329,7 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
             }
         }
     }
+    L.held = held;
     if (bad_point >= 0) {
         msg << "point " << bad_point << ": degenerate " << bad_what;
         err = msg.str();
