@@ -86,11 +86,16 @@ int lskum_mlp_train_step(lskum_mlp* h, const float* feat_dev, const float* targe
 /* Waits for the handle's stream. */
 int lskum_mlp_sync(lskum_mlp* h);
 
-/* GEMM path of the forward pass's five 256-wide layers. Both values select the
- * fused pass on the fifth-generation tensor cores (tcgen05.mma M 128, N 256,
- * K 16 into tensor memory, all layers of 128 samples in one CTA); the call
- * stays for programs that make the choice. A synchronising call returns LSKUM_ERR_TIMEOUT if a wait inside a
- * pass ran out (bounded waits: the kernel sets a flag and returns). */
+/* GEMM path of the forward pass's five 256-wide layers:
+ *   LSKUM_MLP_GEMM_MMA_SYNC  warp-level mma.sync m16n8k16, 64 samples a CTA;
+ *   LSKUM_MLP_GEMM_TCGEN05   fifth-generation tensor cores (the default):
+ *     tcgen05.mma M 128, N 256, K 16 into tensor memory, 128 samples a CTA.
+ * Both take all layers in one launch and accumulate BF16 products in FP32;
+ * results agree to the order of the FP32 sums. The backward pass and the weight
+ * gradients use tcgen05 with either. On tcgen05 a synchronising call returns
+ * LSKUM_ERR_TIMEOUT if a wait inside a pass ran out (bounded waits: the kernel
+ * raises a flag and returns; the context stays usable). Waits for the handle's
+ * stream first. Errors: INVALID_ARG (unknown path). No counterpart in the paper. */
 #define LSKUM_MLP_GEMM_MMA_SYNC 0
 #define LSKUM_MLP_GEMM_TCGEN05 1
 int lskum_mlp_set_gemm(lskum_mlp* h, int path);

@@ -117,7 +117,7 @@ class MLP:
 
     def set_gemm(self, path: int):
         """GEMM path of the forward pass's 256-wide layers (GEMM_MMA_SYNC or
-        GEMM_TCGEN05; both run the fused tcgen05 pass)."""
+        GEMM_TCGEN05, the default)."""
         L._check(self._lib.lskum_mlp_set_gemm(self._h, int(path)), "lskum_mlp_set_gemm")
 
     def close(self):
