@@ -25,7 +25,7 @@ CUDA_SOURCES = ["lskum_kernels.cu", "lskum_kernels_pair.cu", "lskum_kernels_mixe
 HOST_SOURCES = ["lskum_setup.cpp"]
 HEADERS = ["lskum_internal.h", "lskum_kernels.cuh", "math_tables.h", "device_math.cuh",
            "flux_fp64.cuh", "pair_math.cuh", "pair_convert.cuh", "flux_pair.cuh",
-           "pair_tables.h", "flux_fixed.cuh", "fixed_tables.h"]
+           "pair_tables.h", "flux_fixed.cuh", "fixed_tables.h", "flux_mixed.cuh"]
 
 
 def _nvcc() -> str:
