@@ -118,8 +118,11 @@ __device__ __forceinline__ uint32_t entries_pair(const DevGeom& g, const DevGeom
                                                  const int64_t d, const uint32_t cc, const PairPoint& P,
                                                  const int first, const int c, Pf acc[4]) {
     uint32_t left = 0;
-    // for the first look at a step: 1/q4 and 1/(2 sqrt(beta)), floats
+    // for the first look at a step: 1/q4 and 1/(2 sqrt(beta)), floats; no step is
+    // small enough at a point with |S| well beyond the pair form's
     const float iq4 = __fdividef(1.0f, P.qp[3].h), isq = rsqrtf(-2.0f * P.qp[3].h);
+    const float s1 = isq * P.qp[1].h, s2 = isq * P.qp[2].h;
+    const float look = s1 * s1 + s2 * s2 <= 1.1f * kPairMaxS * kPairMaxS ? 1.25f * kPairStep : -1.0f;
     for (int k = first; k < c; k += kClasses) {
         const int64_t at = int64_t(k) * g.stride + d;
         const uint32_t e = g.nbr[at];
@@ -144,7 +147,7 @@ __device__ __forceinline__ uint32_t entries_pair(const DevGeom& g, const DevGeom
         const float fe = f3 * iq4, g1 = f1 - 0.5f * fe * P.qp[1].h, g2 = f2 - 0.5f * fe * P.qp[2].h;
         const float fw = f0 - iq4 * (P.qp[1].h * g1 + P.qp[2].h * g2);
         if (!(fmaxf(fmaxf(fabsf(fe), fabsf(fw) * (kPairStep / kPairStepW)),
-                    isq * fmaxf(fabsf(g1), fabsf(g2))) <= 1.25f * kPairStep)) {
+                    isq * fmaxf(fabsf(g1), fabsf(g2))) <= look)) {
             left |= 1u << k;
             continue;
         }
@@ -205,8 +208,8 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
     static_assert(LANES == 1 || LANES == kClasses, "a thread takes all classes of a point or one");
     // per warp: the large-step entries of one pass of its lanes (owner lane, slot) and their results
     __shared__ uint16_t s_item[BLOCK / 32][32];
-    __shared__ double s_res[BLOCK / 32][4][32];
-    __shared__ double s_R[LANES > 1 ? BLOCK / LANES : 1][4];
+    __shared__ double s_res[BLOCK / 32][4][33];
+    __shared__ double s_R[BLOCK / LANES][4];  // a point's sums
     const int64_t t = (int64_t(blockIdx.x) * BLOCK + threadIdx.x) / LANES;  // (point, condition)
     const int64_t d = t >> g.cshift;
     const uint32_t cc = uint32_t(t) & g.cmask;
@@ -254,7 +257,9 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
 #pragma unroll
     for (int m = 0; m < 4; ++m) R[m] = double(acc[m].h) + double(acc[m].l);
     // entries with large steps: the warp's lanes share them out evenly, 32 a time, and
-    // each point adds its own class by class
+    // a point's are added class by class, its four components by four lanes (by one
+    // lane they were more FP64 instructions than the entries themselves: 56 a pass
+    // of 32 entries, 14 entries a point)
     const int mine = __popc(left);
     int upto = mine;
 #pragma unroll
@@ -263,41 +268,55 @@ __global__ void __launch_bounds__(BLOCK) k_flux_pair(const DevGeom g, const DevG
         if (lane >= o) upto += v;
     }
     const int total = __shfl_sync(0xffffffffu, upto, 31);
-    const int begin = upto - mine;  // positions of the lane's entries: begin .. upto - 1
-    const int end = __shfl_sync(0xffffffffu, upto, lane - part + LANES - 1);  // ... of the point's: .. end - 1
-    int at = begin;
-    uint32_t cls = 0x11111111u;  // the class whose entries are listed next
-    for (int base = 0; base < total; base += 32) {
-        while (left && at < base + 32) {
-            if (LANES == 1)
-                while (!(left & cls)) cls <<= 1;
-            const int k = __ffs(int(LANES == 1 ? left & cls : left)) - 1;
-            s_item[warp][at - base] = uint16_t((lane << 5) | k);
-            left &= ~(1u << k);
-            ++at;
-        }
-        __syncwarp();
-        if (base + lane < total) {
-            const int item = s_item[warp][lane];
-            double c[4];
-            entry_fp64(g, gp, ph, q_in, dq, t - lane / LANES + (item >> 5) / LANES, item & 31, c);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) s_res[warp][m][lane] = c[m];
-        }
-        __syncwarp();
+    constexpr int kWarpPoints = 32 / LANES;
+    double(*const sum)[4] = s_R + warp * kWarpPoints;
+    if (LANES > 1 || total > 0) {
         if (part == 0)
-            for (int p = max(begin, base); p < min(end, base + 32); ++p)
 #pragma unroll
-                for (int m = 0; m < 4; ++m) R[m] += s_res[warp][m][p - base];
-        __syncwarp();
+            for (int m = 0; m < 4; ++m) sum[lane / LANES][m] = R[m];
+        int at = upto - mine;  // positions of the lane's entries: at .. upto - 1
+        const int begin = at;
+        uint32_t cls = 0x11111111u;  // the class whose entries are listed next
+        for (int base = 0; base < total; base += 32) {
+            const int end = min(total, base + 32);
+            while (left && at < end) {
+                if (LANES == 1)
+                    while (!(left & cls)) cls <<= 1;
+                const int k = __ffs(int(LANES == 1 ? left & cls : left)) - 1;
+                s_item[warp][at - base] = uint16_t((lane << 5) | k);
+                left &= ~(1u << k);
+                ++at;
+            }
+            __syncwarp();
+            if (base + lane < total) {
+                const int item = s_item[warp][lane];
+                double c[4];
+                entry_fp64(g, gp, ph, q_in, dq, t - lane / LANES + (item >> 5) / LANES, item & 31, c);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) s_res[warp][m][lane] = c[m];
+            }
+            __syncwarp();
+            const int first = (s_item[warp][0] >> 5) / LANES, last = (s_item[warp][end - 1 - base] >> 5) / LANES;
+            for (int p0 = first; p0 <= last; p0 += 8) {  // eight points a time
+                const int p = p0 + lane / 4, m = lane % 4, own = min(p, kWarpPoints - 1) * LANES;
+                const int from = __shfl_sync(0xffffffffu, begin, own);
+                const int to = __shfl_sync(0xffffffffu, upto, own + LANES - 1);
+                if (p <= last) {
+                    double r = sum[p][m];
+                    for (int i = max(from, base); i < min(to, end); ++i) r += s_res[warp][m][i - base];
+                    sum[p][m] = r;
+                }
+            }
+            __syncwarp();
+        }
+        if (LANES == 1)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) R[m] = sum[lane][m];
     }
     // the stage update: a thread for each point
     int64_t tu = t;
     bool update = live;
     if (LANES > 1) {
-        if (part == 0)
-#pragma unroll
-            for (int m = 0; m < 4; ++m) s_R[threadIdx.x / LANES][m] = R[m];
         __syncthreads();
         tu = int64_t(blockIdx.x) * (BLOCK / LANES) + threadIdx.x;
         update = threadIdx.x < BLOCK / LANES && (tu >> g.cshift) < g.n;
