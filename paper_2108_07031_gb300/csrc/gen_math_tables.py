@@ -49,6 +49,7 @@ mp.mp.dps = 50
 CX_LO, CX_HI, CX_LOG2_INV_W = 0.0, 6.0, 6
 CX_W = 2.0 ** -CX_LOG2_INV_W
 CX_DEG = 6            # degree in z = a - c on [-1/128, 1/128]
+CXT_DEG = 9           # degree in 1/a^2 beyond CX_HI
 EXP_BITS = 8          # 2^(j / 2^EXP_BITS) table
 LOG_BITS = 7          # 2^LOG_BITS mantissa intervals for the log table
 CXF_W, CXF_DEG = 0.25, 5  # FP32 table (mixed precision)
@@ -128,6 +129,15 @@ def main(path=None):
         pieces.append([float(x) for x in C])
         a = hi
 
+    # beyond the pieces: a erfcx(a) in 1/a^2
+    tail = cheb_to_monomial(lambda u: mp.erfc(1 / mp.sqrt(u)) * mp.exp(1 / u) / mp.sqrt(u), mp.mpf(0),
+                            1 / mp.mpf(CX_HI) ** 2, CXT_DEG, mp.mpf(0))
+    zs = np.linspace(0.0, 1 / CX_HI ** 2, 400)[1:]
+    ref = np.array([float(mp.erfc(1 / mp.sqrt(mp.mpf(float(u)))) * mp.exp(1 / mp.mpf(float(u))) /
+                          mp.sqrt(mp.mpf(float(u)))) for u in zs])
+    tail_worst = np.max(np.abs(horner(tail, zs) - ref) / ref)
+    assert tail_worst < 4e-16, ("erfcx tail", tail_worst)
+
     # 2^(j/256) and the split of ln2/256
     n_exp = 1 << EXP_BITS
     tab = [float(mp.mpf(2) ** (mp.mpf(j) / n_exp)) for j in range(n_exp)]
@@ -150,6 +160,12 @@ def main(path=None):
         for c, p in zip(centres, pieces):
             f.write("    {" + f"{c!r}, " + ", ".join(repr(x) for x in p) + "},\n")
         f.write("};\n\n")
+        f.write(f"// a erfcx(a) for a >= {CX_HI} as a polynomial in 1/a^2 (max relative error in double "
+                f"Horner {tail_worst:.2e}).\n")
+        f.write(f"constexpr int kErfcxTailDeg = {CXT_DEG};\n")
+        f.write("__device__ const double kErfcxTail[kErfcxTailDeg + 1] = {\n    " +
+                ",\n    ".join(", ".join(repr(float(x)) for x in tail[k:k + 4]) for k in range(0, len(tail), 4)) +
+                "};\n\n")
         fc, fp, fworst = erfcx_pieces_f32()
         f.write(f"// FP32 erfcx pieces (mixed precision): width {CXF_W}, degree {CXF_DEG}, "
                 f"max relative error {fworst:.2e} in float32 Horner.\n")
