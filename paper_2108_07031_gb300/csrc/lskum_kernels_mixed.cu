@@ -315,7 +315,7 @@ struct MxFrame {
 
 // One entry by the primitive differences: any gamma, any step.
 template <bool G14>
-__device__ __noinline__ float4 entry_prim(const float4 base, const float4 dlt, const float gm1_inv,
+__device__ __forceinline__ float4 entry_prim(const float4 base, const float4 dlt, const float gm1_inv,
                                           const MxFrame f, const uint32_t e, const float ws, const float wn) {
     PrimPair w = prim_pair<G14>(base, dlt, gm1_inv);
     if (f.local) {
@@ -335,6 +335,12 @@ __device__ __noinline__ float4 entry_prim(const float4 base, const float4 dlt, c
         R = make_float4(fmaf(wn, dG[0], R.x), fmaf(wn, dG[2], R.y), fmaf(wn, dG[1], R.z), fmaf(wn, dG[3], R.w));
     }
     return R;
+}
+
+// For gamma = 1.4, where few entries need it: out of the loop's code.
+__device__ __noinline__ float4 entry_prim_g14(const float4 base, const float4 dlt, const MxFrame f,
+                                              const uint32_t e, const float ws, const float wn) {
+    return entry_prim<true>(base, dlt, 2.5f, f, e, ws, wn);
 }
 
 constexpr int kMxClasses = 4;
@@ -444,7 +450,8 @@ __global__ void __launch_bounds__(BLOCK, 896 / BLOCK) k_flux_mx(const DevGeom g,
                 S[2] = fmaf(fw.y, dG[1], S[2]);
                 S[3] = fmaf(wf, dG[3], S[3]);
             } else if (!(dlt.x == 0.f && dlt.y == 0.f && dlt.z == 0.f && dlt.w == 0.f)) {
-                const float4 a = entry_prim<G14>(base, dlt, gm1_inv, f, e, fw.x, fw.y);
+                const float4 a = G14 ? entry_prim_g14(base, dlt, f, e, fw.x, fw.y)
+                                     : entry_prim<false>(base, dlt, gm1_inv, f, e, fw.x, fw.y);
                 S[0] += a.x;
                 S[1] += a.y;
                 S[2] += a.z;
