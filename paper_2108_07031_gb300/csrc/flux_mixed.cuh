@@ -140,9 +140,8 @@ LSKUM_HD float erfc_central_diff(const float m, const float h) {
 LSKUM_HD float half_erfc_f(const float x, const float e) {
     const float a = fabsf(x);
     float hc;
-    if (a <= 6.0f) {
-        const int i = int(a * kErfcxFInvW);
-        const float* c = kErfcxF[i < kErfcxFPieces ? i : kErfcxFPieces - 1];
+    if (a < 6.0f) {
+        const float* c = kErfcxF[int(a * kErfcxFInvW)];
         const float z = a - ldg_f(c);
         float pv = ldg_f(c + 1 + kErfcxFDeg);
 #pragma unroll
