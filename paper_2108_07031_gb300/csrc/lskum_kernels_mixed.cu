@@ -343,6 +343,11 @@ __device__ __noinline__ float4 entry_prim_g14(const float4 base, const float4 dl
     return entry_prim<true>(base, dlt, 2.5f, f, e, ws, wn);
 }
 
+// -x where the sign bit of m is set.
+__device__ __forceinline__ float flip(const float x, const uint32_t m) {
+    return __uint_as_float(__float_as_uint(x) ^ (m & 0x80000000u));
+}
+
 constexpr int kMxClasses = 4;
 // Four threads share a point up to this many (point, condition) pairs: one a
 // point leaves SMs idle there. Microseconds a launch, one thread / four: 5,120
@@ -436,15 +441,16 @@ __global__ void __launch_bounds__(BLOCK, 896 / BLOCK) k_flux_mx(const DevGeom g,
                 }
                 // an entry outside a stencil has weight 0 there
                 float dG[4];
-                float sg = ((e >> kIndexBits) & 3u) == 2u ? -1.f : 1.f, wf = sg * fw.x;
-                mx_diff(w, sg * w.Sxm, sg * w.dSx, w.Sym, w.dSy, dG);
+                uint32_t neg = e << (30 - kIndexBits);  // the sign bit: code 2
+                float wf = flip(fw.x, neg);
+                mx_diff(w, flip(w.Sxm, neg), flip(w.dSx, neg), w.Sym, w.dSy, dG);
                 S[0] = fmaf(wf, dG[0], S[0]);
                 S[1] = fmaf(fw.x, dG[1], S[1]);
                 S[2] = fmaf(wf, dG[2], S[2]);
                 S[3] = fmaf(wf, dG[3], S[3]);
-                sg = ((e >> (kIndexBits + 2)) & 3u) == 2u ? -1.f : 1.f;
-                wf = sg * fw.y;
-                mx_diff(w, sg * w.Sym, sg * w.dSy, w.Sxm, w.dSx, dG);
+                neg = e << (28 - kIndexBits);
+                wf = flip(fw.y, neg);
+                mx_diff(w, flip(w.Sym, neg), flip(w.dSy, neg), w.Sxm, w.dSx, dG);
                 S[0] = fmaf(wf, dG[0], S[0]);
                 S[1] = fmaf(wf, dG[2], S[1]);
                 S[2] = fmaf(fw.y, dG[1], S[2]);
