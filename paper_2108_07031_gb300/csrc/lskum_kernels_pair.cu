@@ -26,9 +26,9 @@ constexpr int kClasses = 4;
 // thread a point leaves SMs idle on a small cloud (5,120 points: 40 blocks),
 // and blocks of 128 points whose entries all have large steps are too large a
 // unit of work to balance; beyond it the four-fold set-up of a point costs more.
-// Microseconds a launch, one thread / four: 5,120 points 156 / 55, 46,080
-// 232 / 170, 150,598 429 / 403, 321,438 638 / 684, 600,138 960 / 1,091.
-constexpr int64_t kSplitPairs = 1 << 18;
+// Microseconds a launch, one thread / four: 5,120 points 141 / 50, 46,080
+// 208 / 151, 150,598 384 / 359, 220,080 457 / 478, 600,138 909 / 1,051.
+constexpr int64_t kSplitPairs = 3 << 16;
 
 // The double of which h + l is the pair and r what it exceeds them by, in units of
 // its last place (lskum_setup.cpp); h and l are finite.
