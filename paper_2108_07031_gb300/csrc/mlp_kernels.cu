@@ -70,11 +70,13 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 // next 64. One warp issues the MMAs, one the copies. The 4-wide output layer
 // is FP32 FMAs on the same BF16 values, in the last epilogue.
 //
-// What bounds it: tanhf, 163,840 a tile on an SM's FP32 pipes (~25 instructions
-// each); the MMAs of a tile are 68 MFLOP x 2, 11 us at the SM's share of the
-// BF16 rate, mostly hidden. A launch per layer wrote and re-read the
+// What bounds it: tanhf first, 163,840 a tile on an SM's FP32 pipes (~25
+// instructions each: 15.5 of the 27 us that a wave of tiles takes); the MMAs of a
+// tile are 69 MFLOP, 5.5 us at the SM's share of the BF16 rate, mostly under it;
+// the rest is the chain through a tile, five layers that each begin with the last
+// one's first 64 columns. A launch per layer wrote and re-read the
 // activations (1.5 KB a row and layer) and filled the chip for 2 us of work:
-// 16,384 samples 176 us a prediction, now 49 (27 in the kernel).
+// 16,384 samples 176 us a prediction, now 46 (27 in the kernel).
 //
 // Operand layout: the no-swizzle K-major canonical form of the matrix
 // descriptors: core matrices of 8 rows x 16 bytes (8 BF16 along K) as 128
@@ -565,7 +567,7 @@ __device__ __forceinline__ void sum_lanes16(float v[16], const int lane) {
 // ------------------------------------------------- fused backward pass
 // The error signals of a 128-row tile from the output to the first layer in one
 // CTA, as k_forward runs forwards (8,192 samples: loss and gradients 659 us with
-// a launch for each layer's product, sum and tanh', now 131): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
+// a launch for each layer's product, sum and tanh', now 114): dZ_4 = (dY W_5) (1 - A_5^2) by FP32 FMAs, then
 // dZ_(l-1) = (dZ_l W_l) (1 - A_l^2) for l = 4..1 with the products on the tensor
 // cores. Stores each layer's dZ in BF16 (the weight gradients' operand), the
 // column sums of the FP32 dZ (the bias gradients; one row of partial sums for
