@@ -102,8 +102,8 @@ cudaError_t dev_alloc(lskum_ctx* c, T** p, size_t count) {
     return e;
 }
 
-template <typename T>
-cudaError_t upload(lskum_ctx* c, const T** dst, const std::vector<T>& src) {
+template <typename T, typename Array>
+cudaError_t upload(lskum_ctx* c, const T** dst, const Array& src) {
     T* p = nullptr;
     cudaError_t e = dev_alloc(c, &p, src.size());
     if (e != cudaSuccess) return e;

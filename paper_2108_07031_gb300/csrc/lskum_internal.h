@@ -2,7 +2,9 @@
 // device kernels (lskum_kernels.cu) and the C ABI (lskum_api.cu).
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -18,6 +20,25 @@ namespace lskum {
 constexpr int kIndexBits = 26;
 constexpr uint32_t kIndexMask = (1u << kIndexBits) - 1u;
 constexpr int kMaxPoints = 1 << kIndexBits;
+
+// An array whose first writes are its filler's, from all threads: a vector writes
+// its zeros first, by one thread (lskum_create at 600,138 points 161 -> 149 ms).
+template <typename T>
+class RawArray {
+public:
+    void allocate(size_t n) {
+        p_.reset(new T[n]);
+        n_ = n;
+    }
+    T& operator[](size_t i) { return p_[i]; }
+    const T* data() const { return p_.get(); }
+    size_t size() const { return n_; }
+    bool empty() const { return n_ == 0; }
+
+private:
+    std::unique_ptr<T[]> p_;
+    size_t n_ = 0;
+};
 
 // Host-side product of lskum_create's set-up, in device point order.
 struct HostLayout {
@@ -46,8 +67,8 @@ struct HostLayout {
     struct Rest4 {
         int8_t v[4];
     };
-    std::vector<Float4> half, weight;
-    std::vector<Rest4> rest;
+    RawArray<Float4> half, weight;
+    RawArray<Rest4> rest;
     bool held = true;
     // FP64 inner sweeps (Eq. 29) split as q_x = (first-order q_x) - sum_j wx_j
     // (hdx_j (qx_j - qx_i) + hdy_j (qy_j - qy_i)), likewise q_y: per slot the

@@ -191,9 +191,9 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
     L.wx.assign(size_t(slots) * S, 0.0);
     L.wy.assign(size_t(slots) * S, 0.0);
     if (pairs) {
-        L.half.assign(size_t(slots) * S, {});
-        L.weight.assign(size_t(slots) * S, {});
-        L.rest.assign(size_t(slots) * S, {});
+        L.half.allocate(size_t(slots) * S);
+        L.weight.allocate(size_t(slots) * S);
+        L.rest.allocate(size_t(slots) * S);
     } else {
         L.hdx.assign(size_t(slots) * S, 0.0);
         L.hdy.assign(size_t(slots) * S, 0.0);
@@ -328,7 +328,22 @@ int build_layout(int64_t n, const double* xy, const double* normals, const int8_
                 for (int m = 0; m < 4; ++m) L.lsum[4 * d + m] += c4[m];
             }
         }
+        if (pairs)
+            for (int k = c; k < slots; ++k) {
+                const size_t at = size_t(k) * S + d;
+                L.half[at] = {};
+                L.weight[at] = {};
+                L.rest[at] = {};
+            }
     }
+    if (pairs)  // the rows' ends
+        for (int k = 0; k < slots; ++k)
+            for (int64_t d = n; d < S; ++d) {
+                const size_t at = size_t(k) * S + d;
+                L.half[at] = {};
+                L.weight[at] = {};
+                L.rest[at] = {};
+            }
     L.held = held;
     if (bad_point >= 0) {
         msg << "point " << bad_point << ": degenerate " << bad_what;
