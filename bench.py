@@ -196,18 +196,18 @@ def _fp64_peak():
 # Per-unit figures of the FP64 path's flux/update kernel (k_flux_pair: float
 # pairs and 64-bit fixed point in place of the FP64 pipe), from one ncu capture
 # of a stage launch on the 2,499,952-point cloud (34,760,611 neighbour entries):
-# 16.872e9 FFMA, 37.185e9 FADD and 10.276e9 FMUL thread instructions (predicated
-# on) = 81.21e9 FP32 flops = 2,336 per neighbour entry, 1,851 FP32 instructions
-# of 2,162 instructions in all (2.3484e9 warp instructions x 32), 0.290e9 FP64
-# instructions (8.3 per entry), and 1,853.5 MB of DRAM traffic = 741.4 bytes per
+# 16.875e9 FFMA, 37.185e9 FADD and 10.251e9 FMUL thread instructions (predicated
+# on) = 81.19e9 FP32 flops = 2,336 per neighbour entry, 1,850 FP32 instructions
+# of 2,149 instructions in all (2.3339e9 warp instructions x 32), 0.288e9 FP64
+# instructions (8.3 per entry), and 1,857.9 MB of DRAM traffic = 743.2 bytes per
 # point. Units of one launch: neighbour entries (flops) and points (bytes); both
 # scale about in proportion with the cloud size (coarser clouds have more of
 # their entries in fixed point). With this instruction mix a saturated FP32 pipe
 # reaches (2 FFMA + FADD + FMUL) / (2 (FFMA + FADD + FMUL)) = 0.631 of the FMA
 # peak.
 FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR = 2336.0
-FLUX_PAIR_INSTR_PER_NEIGHBOUR = 2162.0  # thread instructions, all pipes
-FLUX_DRAM_BYTES_PER_POINT = 741.4
+FLUX_PAIR_INSTR_PER_NEIGHBOUR = 2149.0  # thread instructions, all pipes
+FLUX_DRAM_BYTES_PER_POINT = 743.2
 FLUX_FRAC_CEILING = 0.631
 ISSUE_PEAK = 152 * 4 * 32 * 2.07e9  # thread instructions per second, one a scheduler and clock
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12  # 1.2586
@@ -220,14 +220,14 @@ ALGORITHMIC_BYTES_PER_POINT_ITERATION = 4600.0  # minimal passes, gathers from c
 #   mixed: k_flux_mx, FP32 flops (2 FFMA + FADD + FMUL) per entry; its FP64
 #          epilogue (state update, q-variables) is per point;
 #   split: the four k_flux_part launches and k_stage_split of one stage.
-#   mixed: 0.9051e9 FFMA + 0.9243e9 FMUL + 0.4576e9 FADD = 3.192e9 FP32 flops
-#          = 382.8 per entry (plus 13 FP64 instructions per point), 279.7 MB
-#          of DRAM traffic = 466.1 bytes per point;
+#   mixed: 1.0301e9 FFMA + 0.8576e9 FMUL + 0.4744e9 FADD = 3.392e9 FP32 flops
+#          = 406.8 per entry (plus 13 FP64 instructions per point), 279.8 MB
+#          of DRAM traffic = 466.2 bytes per point;
 #   split: 1.4516e9 DFMA + 0.2950e9 DADD + 0.8724e9 DMUL over the five
 #          launches of a stage = 4.071e9 FP64 flops = 488.2 per entry,
 #          1353.9 MB = 2256 bytes per point.
-FLUX_MX_FP32_FLOPS_PER_NEIGHBOUR = 382.8
-FLUX_MX_DRAM_BYTES_PER_POINT = 466.1
+FLUX_MX_FP32_FLOPS_PER_NEIGHBOUR = 406.8
+FLUX_MX_DRAM_BYTES_PER_POINT = 466.2
 FLUX_SPLIT_FP64_FLOPS_PER_NEIGHBOUR = 488.2
 FLUX_SPLIT_DRAM_BYTES_PER_POINT = 2257.0
 
@@ -508,6 +508,7 @@ def variant_roofline(mixed: bool, split: bool, flux_time, nnz: int, n: int, n_co
     whole step, both from the live CUDA-event times of the timed region."""
     flux_ms, flux_n = flux_time
     launch_s = flux_ms / max(flux_n, 1) * 1e-3
+    captured, counted = "0.6M", "per entry of that launch"
     if mixed:
         kernel, per_entry, per_point = ("k_flux_mx (mixed-precision flux residual + stage update)",
                                         FLUX_MX_FP32_FLOPS_PER_NEIGHBOUR, FLUX_MX_DRAM_BYTES_PER_POINT)
@@ -518,7 +519,9 @@ def variant_roofline(mixed: bool, split: bool, flux_time, nnz: int, n: int, n_co
                                         FLUX_SPLIT_DRAM_BYTES_PER_POINT)
         peak, peak_src = FP64_PEAK_TFLOPS, "derived: 152 SMs x 2 FP64 FMA/clk/SM x 2 flops x 2.07 GHz"
     else:
-        # of small steps throughout; a coarse cloud's entries in fixed point count as theirs
+        captured = "2.5M"
+        counted = ("every entry as a small step's, in float pairs; a large one's takes fixed point, so "
+                   "a cloud of 0.6M points, with a quarter of them, reads high")
         kernel, per_entry, per_point = ("k_flux_pair (flux residual + stage update, FP64 path in float pairs)",
                                         FLUX_PAIR_FP32_FLOPS_PER_NEIGHBOUR, FLUX_DRAM_BYTES_PER_POINT)
         peak, peak_src = FP32_PEAK_TFLOPS, "derived: 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz"
@@ -529,9 +532,9 @@ def variant_roofline(mixed: bool, split: bool, flux_time, nnz: int, n: int, n_co
     layout = layout_bytes_per_point_iteration(mixed, nnz / n)
     return {"kernel": kernel, "bound": "alu", "unit": "TFLOP/s", "achieved": achieved,
             "peak": peak, "frac": achieved / peak if achieved else None, "peak_source": peak_src,
-            "launch_ms": launch_s * 1e3,
+            "launch_ms": launch_s * 1e3, "achieved_note": counted,
             "traffic": per_point * n * n_cond if per_point else None,
-            "traffic_note": "ncu dram bytes of a 0.6M-point launch, scaled by points x conditions",
+            "traffic_note": f"ncu dram bytes of a {captured}-point launch, scaled by points x conditions",
             "hbm_frac_of_measured_whole_step": {
                 "algorithmic": ALGORITHMIC_BYTES_PER_POINT_ITERATION * n * n_cond / step_s / hbm,
                 "layout": layout * n * n_cond / step_s / hbm,

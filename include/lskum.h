@@ -59,7 +59,8 @@ extern "C" {
 
 /* Precision modes. */
 #define LSKUM_FP64 0  /* every step in FP64, or to its accuracy in float pairs and
-                         64-bit fixed point (the fluxes of gamma = 1.4) */
+                         64-bit fixed point (the fluxes of gamma = 1.4 on clouds whose
+                         neighbours lie 2^-29 to 2^31 apart; FP64 on others) */
 #define LSKUM_MIXED 1 /* FP32 stencil, least-squares and split-flux arithmetic (in
                          difference form, on q stored as float pairs); q-variables
                          in float pairs; FP64 state accumulation, LS determinants,

@@ -135,7 +135,7 @@ LSKUM_HD float erfc_central_diff(const float m, const float h) {
 }
 
 // erfc(x)/2 given e = exp(-x^2): e erfcx(|x|)/2 from the FP32 erfcx pieces
-// (width 1/4, degree 5, 1.2e-7 relative) for |x| <= 6, then 1 minus it for
+// (width 1/4, degree 5, 1.2e-7 relative) for |x| < 6, then 1 minus it for
 // x < 0; the exponential is the one the split flux needs for B anyway.
 LSKUM_HD float half_erfc_f(const float x, const float e) {
     const float a = fabsf(x);

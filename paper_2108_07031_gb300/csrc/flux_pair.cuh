@@ -34,8 +34,9 @@ namespace lskum {
 // Largest step of beta (relative) and S; of ln(rho beta^(5/2)), which is several
 // times the primitive variables' and enters dG only to first order. Measured
 // against binary128, 2-norm of the residual's error over the FP64 kernel's: at
-// 1/64 0.3-0.8 on developed states of 2,000-150,000 points, 0.8-1.1 on a flow
-// 300 iterations from the free stream; at 1/40 up to 1.9 on the latter.
+// 1/64 0.46-0.85 on perturbed states of 600 and 1,500 points (eight to twelve seeds),
+// 0.2-0.9 on others up to 46,080, 0.65-1.05 on eight flows 100 to 1,000 iterations
+// from the free stream (one component of one 1.18); at 1/40 up to 1.9 on the latter.
 constexpr float kPairStep = 1.0f / 64.0f;
 constexpr float kPairStepW = 4.0f * kPairStep;
 constexpr float kPairMaxS = 5.9f;          // |S| inside the Phi table

@@ -351,15 +351,15 @@ __device__ __forceinline__ float flip(const float x, const uint32_t m) {
 constexpr int kMxClasses = 4;
 // Four threads share a point up to this many (point, condition) pairs: one a
 // point leaves SMs idle there. Microseconds a launch, one thread / four: 5,120
-// points 36 / 17, 46,080 39 / 27, 79,948 42 / 33, 150,598 53 / 54.
+// points 35 / 17, 46,080 38 / 27, 79,948 42 / 33, 150,598 54.8 / 55.1.
 constexpr int64_t kMxSplitPairs = 1 << 17;
 // The same for the sweeps, whose set-up weighs more: the iteration of 5,120
 // points takes 127 / 120 us, of 30,070 155 / 150; a sweep of 79,948 12 / 16.
 constexpr int64_t kMxSplitSweep = 1 << 15;
 
-// Issue-bound (75 % of the slots at 0.6M points, FP64 pipe 10 %: 144 us a launch;
+// Issue-bound (76 % of the slots at 0.6M points, FP64 pipe 15 %: 145 us a launch;
 // with the primitive differences, and q and every conversion on the FP64 pipe,
-// 172 us and 57 %; 2.5M points 608 -> 520). Each neighbour entry's stream loads
+// 172 us and 57 %; 2.5M points 608 -> 530). Each neighbour entry's stream loads
 // (packed word, FP32 constants) are issued one entry ahead, so that only the
 // gathers they index are waited on; registers capped at 72. A point's
 // entries are summed by class (slot mod kMxClasses) and the classes in order, by

@@ -4,13 +4,13 @@
 // What bounds it: instruction issue (66 % of the slots at 2.5M points). A
 // split-flux difference costs 225 FP64 instructions per neighbour entry, and the
 // FP64 pipe issues two per clock and SM where the FP32 pipes issue 128. The pair
-// form takes about 1,850 FP32 instructions: at 2.5M points 2.89 ms a launch
-// instead of 14.75, at 0.6M 0.95 instead of 3.58, at 5,120 0.055 instead of
+// form takes about 1,850 FP32 instructions: at 2.5M points 2.88 ms a launch
+// instead of 14.75, at 0.6M 0.91 instead of 3.58, at 5,120 0.050 instead of
 // 0.148. Entries that are not the pair form's (large steps: a quarter at 0.6M,
-// most at 5,120) are noted in a bit mask and evaluated after the loop in 64-bit
-// fixed point (flux_fixed.cuh; by k_flux's FP64 formulas the launches took 0.99
-// and 0.068), a warp's entries spread evenly over its lanes; the stage update,
-// the next stage's q-variables and the residue stay FP64.
+// most at 5,120) are noted in a bit mask and evaluated after the loop from the
+// doubles, in 64-bit fixed point (flux_fixed.cuh), a warp's entries spread evenly
+// over its lanes; the stage update, the next stage's q-variables and the residue
+// stay FP64.
 
 #include "flux_fixed.cuh"
 #include "flux_fp64.cuh"
@@ -59,7 +59,7 @@ __device__ __noinline__ void general_diff(const double* tj, const double* t0, co
 }
 
 // ws dGs + wn dGn of entry k of point d to FP64's accuracy, in the point's frame:
-// what k_flux adds for that entry. 64 FP64 instructions and some 1,700 on the
+// what k_flux adds for that entry. 48 FP64 instructions and some 1,700 on the
 // integer pipe (flux_fixed.cuh), where k_flux's formulas take 230 FP64 ones.
 __device__ __forceinline__ void entry_fp64(const DevGeom& g, const DevGeomPair& gp, const Physics& ph,
                                            const V4* __restrict__ q_in, const V8* __restrict__ dq,
