@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(BLOCK) k_ls_inner_mx4(const DevGeom g, const D
 }
 
 __device__ __forceinline__ QHL split_hl(const V4& q) {
-    const Pf a = split_pair(q.a), b = split_pair(q.b), c = split_pair(q.c), d = split_pair(q.d);
+    const Pf a = nearest_pair(q.a), b = nearest_pair(q.b), c = nearest_pair(q.c), d = nearest_pair(q.d);
     return QHL{make_float4(a.h, b.h, c.h, d.h), make_float4(a.l, b.l, c.l, d.l)};
 }
 

@@ -26,7 +26,7 @@ LSKUM_HD double dvalue(uint64_t u) {
 }
 
 #ifdef __CUDACC__
-// x as a pair: the leading 24 bits truncated, the other 29 rounded to a float.
+// x as a pair to 2^-48: the leading 24 bits truncated, the other 29 rounded to a float.
 // Integer operations only (the conversions between FP64 and FP32 run at the
 // FP64 pipe's rate). |x| below 2^-74 gives zero, above 2^127 or not finite NaN.
 __device__ __forceinline__ Pf split_pair(const double x) {
@@ -44,6 +44,12 @@ __device__ __forceinline__ Pf split_pair(const double x) {
     return r;
 }
 #endif
+
+// x as the nearest pair, to 2^-49: where the conversions' rate does not matter.
+LSKUM_HD Pf nearest_pair(const double x) {
+    const float h = float(x);
+    return {h, float(x - double(h))};
+}
 
 // The double equal to a float, infinities and NaN included, by integer
 // operations; subnormals give zero.
